@@ -3,8 +3,9 @@
 // audio condition tokens (cross-attention).
 //
 // Flash-style forward on the 5th-generation tensor cores.  One CTA per
-// (two 128-query tiles, head), 12 warps, with the two tiles in ping-pong so
-// that one tile's softmax runs while the tensor cores work on the other:
+// (two 128-query tiles, head), or a cluster of 2, 4 or 8 CTAs that split its key
+// blocks, 12 warps, with the two tiles in ping-pong so that one tile's softmax
+// runs while the tensor cores work on the other:
 //   warp 0      TMA producer: both Q tiles once, then 128-key blocks K_0, V_0,
 //               K_1, V_1, ... (128-byte swizzle, 64-column boxes) into a ring
 //               shared by K and V (5 slots for d = 128);
@@ -37,7 +38,8 @@ constexpr int THREADS = 384;   // 4 control warps + 2 softmax warpgroups
 constexpr uint32_t TMEM_COLS = 512;   // S0, S1, O0, O1
 constexpr uint32_t O_COL = 256;
 constexpr int ATOM_BYTES = 128 * 128;   // one [128 rows x 64 bf16] 128B-swizzled box
-// up to this many keys: the persistent kernel below (measured at 6552 queries,
+// up to this many keys, unless the keys are split over a cluster (choose_splits):
+// the persistent kernel below (measured at 6552 queries,
 // 40 heads of 128: faster by 8% at 1280 keys, slower by 3% at 2560 and by 7% at
 // 4096, where the one-shot kernel's waves already hide its fixed costs)
 constexpr int kItemsMaxKeys = 2048;
@@ -61,7 +63,84 @@ struct AttnParams {
     int *err;
 };
 
+// The results of the CTAs of a cluster, each over its own key blocks, summed
+// through distributed shared memory: with the rows' maxima m_r and sums l_r of
+// every CTA, O = sum_r 2^(m_r - m) O_r / sum_r 2^(m_r - m) l_r, m = max_r m_r.
+// m_r and l_r go to the tile's finished Q buffer.  Each thread scales its row of
+// this CTA's O by 2^(m_own - m) / sum and stages it in fp32 over the ring (free:
+// every MMA is done after the first barrier); then CTA r adds rows [256 r / S, 256 (r + 1) / S) of every CTA in
+// rank order, rounds and stores them.  Three cluster barriers, which the
+// control warps pass too; a CTA that gave up passes them without its results.
+template <int DH, int S>
+ECHO_DEV void sum_split_rows(const AttnParams &p, uint32_t stage_addr, int split, int q0, int h) {
+    constexpr int LPR = DH / 4;                 // lanes per row, one 16-byte chunk each
+    constexpr int RPW = 32 / LPR;               // rows per warp-wide load
+    constexpr int ROWS = TILES * BM / S;        // rows of this CTA
+    const int warp = ((int)threadIdx.x >> 5) - 4, lane = threadIdx.x & 31;
+    uint32_t base[S];
+#pragma unroll
+    for (int r = 0; r < S; ++r) base[r] = mapa_shared(stage_addr, (uint32_t)r);
+#pragma unroll 2
+    for (int i = warp * RPW; i < ROWS; i += 8 * RPW) {
+        const int row = split * ROWS + i + lane / LPR, cc = lane % LPR;
+        const uint32_t off = (uint32_t)(row * DH * 4 + ((cc ^ (row & 7)) * 16));
+        float4 v[S];
+#pragma unroll
+        for (int r = 0; r < S; ++r) v[r] = ld_shared_cluster_f4(base[r] + off);
+#pragma unroll
+        for (int r = 1; r < S; ++r) {
+            v[0].x += v[r].x; v[0].y += v[r].y; v[0].z += v[r].z; v[0].w += v[r].w;
+        }
+        const int grow = q0 + row;
+        if (grow < p.M)
+            *reinterpret_cast<uint2 *>(p.O + (int64_t)grow * p.ldo + h * DH + 4 * cc) =
+                make_uint2(pack_bf16(v[0].x, v[0].y), pack_bf16(v[0].z, v[0].w));
+    }
+}
+
 template <int DH>
+ECHO_DEV void combine_splits(const AttnParams &p, uint8_t *stage, float2 *own_ml, uint32_t o_tmem,
+                             int row, float m_own, float l_own, bool ok, int splits, int split,
+                             int q0, int h) {
+    static_assert(TILES * BM * DH * 4 <= Cfg<DH>::RING * Cfg<DH>::SLOT_BYTES, "staged over the ring");
+    if (l_own == 0.f) m_own = -INFINITY;
+    *own_ml = make_float2(m_own, l_own);
+    __syncwarp();
+    cluster_sync_all();
+    const uint32_t ml_addr = smem_u32(own_ml);
+    float m = m_own;
+    for (int r = 0; r < splits; ++r)
+        m = fmaxf(m, ld_shared_cluster_f2(mapa_shared(ml_addr, (uint32_t)r)).x);
+    float l = 0.f;
+    for (int r = 0; r < splits; ++r) {
+        const float2 ml = ld_shared_cluster_f2(mapa_shared(ml_addr, (uint32_t)r));
+        l += ex2_approx(ml.x - m) * ml.y;
+    }
+    const float f = ex2_approx(m_own - m) / l;
+    if (ok) {   // warp-uniform
+#pragma unroll
+        for (int c = 0; c < DH / 32; ++c) {
+            uint32_t o[32];
+            tmem_ld32(o_tmem + 32 * c, o);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                *reinterpret_cast<float4 *>(stage + row * DH * 4 + (((8 * c + i) ^ (row & 7)) * 16)) =
+                    make_float4(__uint_as_float(o[4 * i]) * f, __uint_as_float(o[4 * i + 1]) * f,
+                                __uint_as_float(o[4 * i + 2]) * f, __uint_as_float(o[4 * i + 3]) * f);
+        }
+    }
+    __syncwarp();
+    cluster_sync_all();
+    const uint32_t stage_addr = smem_u32(stage);
+    if (splits == 2) sum_split_rows<DH, 2>(p, stage_addr, split, q0, h);
+    else if (splits == 4) sum_split_rows<DH, 4>(p, stage_addr, split, q0, h);
+    else sum_split_rows<DH, 8>(p, stage_addr, split, q0, h);
+    __syncwarp();
+    cluster_sync_all();   // no CTA leaves while another may still read its rows
+}
+
+template <int DH, bool SPLIT>
 __global__ void __launch_bounds__(THREADS, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
@@ -83,8 +162,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int h = blockIdx.y;
-    const int q0 = blockIdx.x * (TILES * BM);
-    const int nb = (p.L + BN - 1) / BN;
+    // the CTAs of a cluster share the queries and split the key blocks
+    const int splits = SPLIT ? (int)cluster_nctarank() : 1, split = SPLIT ? (int)cluster_ctarank() : 0;
+    const int q0 = ((int)blockIdx.x / splits) * (TILES * BM);
+    const int nb_all = (p.L + BN - 1) / BN;
+    const int kb0 = SPLIT ? (int)((int64_t)nb_all * split / splits) : 0;   // this CTA's first block
+    const int nb = SPLIT ? (int)((int64_t)nb_all * (split + 1) / splits) - kb0 : nb_all;
 
     if (threadIdx.x == 0) {
         mbar_init(&q_full, 1);
@@ -127,7 +210,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             const CUtensorMap *m = (li & 1) ? &tmV : &tmK;
             for (int a = 0; a < C::ATOMS; ++a)
                 tma_load_2d(Ring + slot * C::SLOT_BYTES + a * ATOM_BYTES, m, &ring_full[slot],
-                            x0 + 64 * a, (li >> 1) * BN);
+                            x0 + 64 * a, (kb0 + (li >> 1)) * BN);
             issued = li + 1;
         }
         if (*abort_v) {  // let this CTA's copies land before it exits
@@ -250,6 +333,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             mbar_wait(&drain, 0, abort_v, nullptr, 100000000ull);
         }
     }
+    if constexpr (SPLIT) {   // the three cluster barriers of combine_splits
+        __syncwarp();
+        cluster_sync_all();
+        cluster_sync_all();
+        cluster_sync_all();
+    }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 224;" ::: "memory");
         // ---------------- softmax / correction / epilogue of tile t ----------------
@@ -266,7 +355,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             if (!ok) break;
             tc_fence_after();
             // the whole S row of this block in registers (one TMEM round trip)
-            const int kvalid = p.L - j * BN;                 // keys of this block that exist
+            const int kvalid = p.L - (kb0 + j) * BN;         // keys of this block that exist
             float sv[BN];
 #pragma unroll
             for (int c = 0; c < BN / 32; ++c)
@@ -313,7 +402,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 f2_unpack(f2_add(f2_add(acc2[0], acc2[1]), f2_add(acc2[2], acc2[3])), a0, a1);
                 return a0 + a1;
             };
-            if (j == 0) m_used = block_max() * sl2;
+            if (j == 0) {
+                m_used = block_max() * sl2;
+                // a CTA whose first keys all score -inf adds nothing to the sums
+                // of the others instead of NaN
+                if (SPLIT && m_used == -INFINITY) m_used = 0.f;
+            }
             float bsum = exp_pass();
             const bool redo = !(bsum <= 1.8446744e19f);     // > 2^64, inf or NaN
             if (__any_sync(0xffffffffu, redo)) {              // rare: warp-uniform slow path
@@ -349,8 +443,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             if (lane == 0) mbar_arrive(&p_full[t]);
         }
         if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&pv_done[t], 0, abort_v, p.err));
-        if (ok) {
-            tc_fence_after();
+        if (ok) tc_fence_after();
+        if constexpr (SPLIT) {
+            // the rows' maxima and sums in the tile's Q, the scaled rows over the ring
+            combine_splits<DH>(p, Ring,
+                               reinterpret_cast<float2 *>(Qs + t * C::Q_BYTES) + quad * 32 + lane,
+                               tmem + lane_base + o_col, t * BM + quad * 32 + lane, m_used, l, ok,
+                               splits, split, q0, h);
+        } else if (ok) {
             const float inv = 1.f / l;
             // The warp's 32 rows of O go through its quarter of Q_t (free now:
             // every MMA that read Q_t is done) and leave in whole row segments,
@@ -879,17 +979,81 @@ echo_status launch_items_dh(const void *Q, int64_t ldq, const void *K, const voi
     }
 }
 
+constexpr int kSplitMax = 8;   // CTAs of a cluster (portable size)
+
+// attn_tc_kernel may take its dynamic shared memory (once per device)
 template <int DH>
-echo_status launch_dh(const void *Q, int64_t ldq, const void *K, const void *V, int64_t ldkv, int M,
-                      int L, int H, void *O, int64_t ldo, cudaStream_t st) {
+void raise_smem_cap() {
     static int attr_done[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-        cudaFuncSetAttribute(attn_tc_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(attn_tc_kernel<DH, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             Cfg<DH>::SMEM);
+        cudaFuncSetAttribute(attn_tc_kernel<DH, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              Cfg<DH>::SMEM);
         attr_done[dev] = 1;
     }
+}
+
+// CTAs of attn_tc_kernel<DH, true> that run at once in clusters of `splits`, on the
+// current device (one CTA per SM; clusters of 4 and 8 leave a few SMs idle)
+template <int DH>
+int split_slots(int splits) {
+    static int slots[64][kSplitMax + 1] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    int &n = slots[dev][splits];
+    if (!n) {   // a benign race computes the same value twice
+        if (splits == 1) return n = num_sms();
+        raise_smem_cap<DH>();
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(splits * num_sms()), 1, 1);
+        cfg.blockDim = dim3(THREADS, 1, 1);
+        cfg.dynamicSmemBytes = Cfg<DH>::SMEM;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)splits;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int c = 0;
+        if (cudaOccupancyMaxActiveClusters(&c, attn_tc_kernel<DH, true>, &cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            c = 0;
+        }
+        n = c > 0 ? c * splits : -1;
+    }
+    return n > 0 ? n : 0;
+}
+
+// Over how many CTAs to split the keys of one (tile pair, head), so that few
+// active latents still fill the SMs: the fewest key-block times (1.2 us),
+// counted as waves of CTAs times the blocks of one CTA plus its fixed cost
+// (set-up and epilogue 4; with the sum over the cluster 7).  Measured, one CTA
+// against the split chosen: 389 queries x 7801 keys, 16 heads of 64: 80.7 ->
+// 29.6 us (4); 130 x 2000 x 6 heads of 64: 23.1 -> 10.8 us (8); 600 x 2000 x 16
+// heads of 64: 23.7 -> 16.9 us (2); 3198 x 63960 x 40 heads of 128 (3.4 waves):
+// 2.71 -> 2.60 ms under the power cap (2).  At 1560 x 7800 x 16 (0.74 waves) two take
+// 89 us against 76 and the rule stays at one.
+template <int DH>
+int choose_splits(int64_t items, int nb) {
+    int best = 1;
+    int64_t best_cost = INT64_MAX;
+    for (int sp = 1; sp <= kSplitMax && sp <= nb; sp *= 2) {
+        const int slots = split_slots<DH>(sp);
+        if (!slots) continue;
+        const int64_t waves = (items * sp + slots - 1) / slots;
+        const int64_t cost = waves * ((nb + sp - 1) / sp + (sp == 1 ? 4 : 7));
+        if (cost < best_cost) { best_cost = cost; best = sp; }
+    }
+    return best;
+}
+
+template <int DH>
+echo_status launch_dh(const void *Q, int64_t ldq, const void *K, const void *V, int64_t ldkv, int M,
+                      int L, int H, int splits, void *O, int64_t ldo, cudaStream_t st) {
+    raise_smem_cap<DH>();
     CUtensorMap tq, tk, tv;
     const uint64_t cols = (uint64_t)H * DH;
     if (!echo::make_tmap_bf16(&tq, Q, (uint64_t)M, cols, (uint64_t)ldq, BM) ||
@@ -903,9 +1067,26 @@ echo_status launch_dh(const void *Q, int64_t ldq, const void *K, const void *V, 
     p.O = static_cast<__nv_bfloat16 *>(O);
     p.ldo = ldo;
     p.err = echo::device_error_ptr();
-    dim3 grid((M + TILES * BM - 1) / (TILES * BM), H);
+    const int ntp = (M + TILES * BM - 1) / (TILES * BM);
+    if (splits == 1) {
+        echo::LaunchScope ls(ECHO_K_ATTENTION, M, L, (int64_t)H * DH, st);
+        attn_tc_kernel<DH, false><<<dim3(ntp, H), THREADS, Cfg<DH>::SMEM, st>>>(tq, tk, tv, p);
+        return echo::last_launch_status();
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(ntp * splits), (unsigned)H, 1);
+    cfg.blockDim = dim3(THREADS, 1, 1);
+    cfg.dynamicSmemBytes = Cfg<DH>::SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)splits;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
     echo::LaunchScope ls(ECHO_K_ATTENTION, M, L, (int64_t)H * DH, st);
-    attn_tc_kernel<DH><<<grid, THREADS, Cfg<DH>::SMEM, st>>>(tq, tk, tv, p);
+    if (cudaLaunchKernelEx(&cfg, attn_tc_kernel<DH, true>, tq, tk, tv, p) != cudaSuccess)
+        return ECHO_ERR_CUDA;
     return echo::last_launch_status();
 }
 
@@ -917,12 +1098,15 @@ echo_status launch_attention(const void *Q, int64_t ldq, const void *K, const vo
                              int32_t M, int32_t L, int32_t H, int32_t d, void *O, int64_t ldo,
                              cudaStream_t st) {
     if (M <= 0) return ECHO_OK;
-    if (L <= kItemsMaxKeys) {   // short key sets: the persistent kernel
+    const int64_t items = ((int64_t)M + TILES * BM - 1) / (TILES * BM) * H;
+    const int nb = (L + BN - 1) / BN;
+    const int splits = d == 64 ? choose_splits<64>(items, nb) : choose_splits<128>(items, nb);
+    if (L <= kItemsMaxKeys && splits == 1) {   // short key sets: the persistent kernel
         if (d == 64) return launch_items_dh<64>(Q, ldq, K, V, ldkv, M, L, H, O, ldo, st);
         return launch_items_dh<128>(Q, ldq, K, V, ldkv, M, L, H, O, ldo, st);
     }
-    if (d == 64) return launch_dh<64>(Q, ldq, K, V, ldkv, M, L, H, O, ldo, st);
-    return launch_dh<128>(Q, ldq, K, V, ldkv, M, L, H, O, ldo, st);
+    if (d == 64) return launch_dh<64>(Q, ldq, K, V, ldkv, M, L, H, splits, O, ldo, st);
+    return launch_dh<128>(Q, ldq, K, V, ldkv, M, L, H, splits, O, ldo, st);
 }
 
 }  // namespace echo

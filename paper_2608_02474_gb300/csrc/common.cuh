@@ -203,6 +203,12 @@ ECHO_DEV uint32_t cluster_ctarank() {
     return r;
 }
 
+ECHO_DEV uint32_t cluster_nctarank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+
 // Address of the same shared-memory location in CTA `rank` of this cluster.
 ECHO_DEV uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
     uint32_t r;
@@ -214,6 +220,24 @@ ECHO_DEV uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
 ECHO_DEV int ld_shared_cluster_s32(uint32_t cluster_addr) {
     int v;
     asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
+    return v;
+}
+
+ECHO_DEV float2 ld_shared_cluster_f2(uint32_t cluster_addr) {
+    float2 v;
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];"
+                 : "=f"(v.x), "=f"(v.y)
+                 : "r"(cluster_addr)
+                 : "memory");
+    return v;
+}
+
+ECHO_DEV float4 ld_shared_cluster_f4(uint32_t cluster_addr) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(cluster_addr)
+                 : "memory");
     return v;
 }
 

@@ -1,0 +1,72 @@
+"""Attention with the keys split over a cluster of CTAs, against the oracle.
+
+The rule takes 2, 4 or 8 CTAs per (tile pair, head) when the pairs alone leave
+SMs idle; the sizes below fall on every width, with key blocks that do not
+divide evenly, a last block of one key and ragged query tiles.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+import oracle                                      # noqa: E402
+from synth import generate as G                    # noqa: E402
+
+F32 = np.float32
+
+
+@pytest.fixture(scope="module")
+def ec():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_2608_02474_gb300 import echocache
+    return echocache
+
+
+def bf(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a)).to("cuda", torch.bfloat16)
+
+
+def check(ec, Q, KV, H, d):
+    D = H * d
+    kvd = bf(KV)
+    out = ec.echo_attention(bf(Q), kvd[:, :D], kvd[:, D:], H, d).float().cpu().numpy()
+    ref = oracle.block.mha(Q.astype(np.float64), KV[:, :D].astype(np.float64),
+                           KV[:, D:].astype(np.float64), H)
+    # P and the result in bf16 (2^-9 each), sums in fp32: the bar of the one-CTA form
+    rel = np.abs(out - ref).max(axis=1) / np.abs(ref).max(axis=1)
+    assert rel.max() <= 2e-2 and np.abs(out - ref).sum() / np.abs(ref).sum() <= 5e-3
+    assert ec.echo_get_device_error() == 0
+
+
+@pytest.mark.parametrize("M,L,H,d", [
+    (1, 1025, 1, 64),        # 8 CTAs, 9 blocks, the last of one key
+    (257, 1025, 1, 128),     # two tile pairs, the second of one row
+    (130, 7801, 2, 64),      # 8 CTAs, 61 blocks: 7 or 8 each
+    (389, 2000, 16, 64),     # 4 CTAs
+    (256, 2500, 19, 128),    # 4 or 8 CTAs, whole tiles
+    (600, 1999, 16, 128),    # 2 CTAs
+    (1100, 900, 12, 64),     # 2 CTAs, 8 blocks
+])
+def test_attention_split_keys(ec, M, L, H, d):
+    D = H * d
+    check(ec, G.random_rows(M, D, seed=M + d, scale=1.5),
+          G.random_rows(L, 2 * D, seed=L + d, scale=1.5), H, d)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("lo,hi", [(0, 300), (3000, 4000), (1900, 2100)])
+def test_attention_split_maxima_differ(ec, d, lo, hi):
+    """Keys lo..hi hold nearly all of the weight: the CTAs' maxima lie far
+    apart, and all but one or two of them contribute next to nothing."""
+    H, M, L = 2, 150, 4000
+    D = H * d
+    g = np.random.default_rng(d)
+    Q = np.full((M, D), 2.0, dtype=F32) + g.standard_normal((M, D)).astype(F32) * F32(0.05)
+    K = g.standard_normal((L, D)).astype(F32) * F32(0.1)
+    K[lo:hi] += F32(3.0)
+    V = g.standard_normal((L, D)).astype(F32)
+    Q, K, V = (G.to_bf16_values(a) for a in (Q, K, V))
+    check(ec, Q, np.concatenate([K, V], axis=1), H, d)
