@@ -2,22 +2,27 @@
 // projections, FFN on the active latents; Sec. 3.3) on the 5th-generation
 // tensor cores:  out = act(A W^T + bias) + resid.
 //
-// Persistent CTA pairs: a cluster of two CTAs on two SMs walks 256 x 256 output
-// tiles in a banded order and computes each with tcgen05.mma.cta_group::2
-// (M 256, N 256, K 16): the even CTA holds rows 0..127 of the tile, the odd CTA
-// rows 128..255, and each holds one 128-row half of the W tile, so each SM loads
-// 32 KB per 64-deep k-block instead of the 48 KB of a one-SM 128 x 256 tile.
-// 8 warps per CTA:
-//   warp 0      TMA producer: the CTA's A [128 x 64] and W-half [128 x 64] bf16
-//               tiles, 128-byte swizzle, into a 6-stage ring (32 KB per stage);
+// Persistent CTA pairs: a cluster of two CTAs on two SMs walks 256 x BN output
+// tiles (BN 256, or 128 for small outputs) in a banded order and computes each
+// with tcgen05.mma.cta_group::2 (M 256, N BN, K 16): the even CTA holds rows
+// 0..127 of the tile, the odd CTA rows 128..255, and each holds one half of the W
+// tile, so each SM loads 32 KB per 64-deep k-block (BN 256) instead of the 48 KB
+// of a one-SM 128 x 256 tile.  12 warps per CTA:
+//   warp 0      TMA producer: the CTA's A [128 x 64] and W-half [BN/2 x 64] bf16
+//               tiles, 128-byte swizzle, into a ring of 6 (BN 256) or 8 stages;
 //               both CTAs' copies complete their bytes on the even CTA's barrier;
 //   warp 1      (even CTA) one elected lane issues the pair MMAs into one of two
-//               256-column fp32 accumulators (the same columns in both CTAs) and
+//               BN-column fp32 accumulators (the same columns in both CTAs) and
 //               commits each stage back to both producers, so the epilogue of one
 //               tile overlaps the main loop of the next;
-//   warp 2      allocates / frees the 512 tensor-memory columns of the pair;
-//   warps 4..7  epilogue, in each CTA: tcgen05.ld 32 columns at a time (warp w
-//               reads TMEM lanes 32 (w mod 4) ..), adds bias, GELU, residual, stores.
+//   warp 2      allocates / frees the tensor-memory columns of the pair;
+//   warps 4..11 epilogue, in each CTA (warp w reads TMEM lanes 32 (w mod 4) .. and
+//               one half of the columns): 32 x 32 blocks through shared memory, so
+//               that bias, GELU, residual and the stores run on whole row segments
+//               (8 lanes a row).  A row per lane instead, with four warps, took as
+//               long as the main loop of a 1024-deep tile: 1560 x 1024 x 1024 with
+//               an fp32 residual 19.1 -> 10.6 us, 20000 x 768 x 768 94 -> 43 us,
+//               6552 x 5120 x 5120 221 -> 196 us.
 // Every mbarrier wait is bounded (ECHO_ERR_TIMEOUT); a CTA that gives up lets its
 // copies land and drains its MMAs before it frees tensor memory, and a cluster
 // barrier keeps either CTA from leaving while the other may still reach it.
@@ -26,15 +31,23 @@
 
 namespace {
 
-constexpr int BM = 128, BN = 256, BK = 64, STAGES = 6;   // BM: rows per CTA of a pair tile
+constexpr int BM = 128, BK = 64;             // BM: rows per CTA of a pair tile
 constexpr int A_BYTES = BM * BK * 2;         // 16 KB
-constexpr int HB_BYTES = (BN / 2) * BK * 2;  // half of a W tile: 16 KB
-constexpr int STAGE_BYTES = A_BYTES + HB_BYTES;
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;  // + alignment slack
-constexpr int THREADS = 256;
-constexpr uint32_t TMEM_COLS = 512;   // two 256-column accumulators
-constexpr int GROUP_N = 16;            // N tiles per raster band
-constexpr uint32_t IDESC = idesc_bf16_f32(2 * BM, BN);
+constexpr int EPI_WARPS = 8;
+constexpr int STG_BYTES = 32 * 32 * 4;       // one 32 x 32 fp32 block per epilogue warp
+constexpr int THREADS = 128 + 32 * EPI_WARPS;
+constexpr int BAND_COLS = 4096;              // output columns per raster band
+
+template <int BN>
+struct Cfg {
+    static constexpr int HB_BYTES = (BN / 2) * BK * 2;   // half of a W tile
+    static constexpr int STAGE_BYTES = A_BYTES + HB_BYTES;
+    static constexpr int STAGES = BN == 256 ? 6 : 8;
+    static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EPI_WARPS * STG_BYTES + 1024;
+    static constexpr uint32_t TMEM_COLS = 2 * BN;        // two accumulators
+    static constexpr int GROUP_N = BAND_COLS / BN;       // N tiles per raster band
+    static constexpr uint32_t IDESC = idesc_bf16_f32(2 * BM, BN);
+};
 
 // EPI_ROWAMAX: also fold max |v| of each bf16 output row into row_amax (fp32
 // bits, atomic max over the row's column tiles; a NaN beats every number)
@@ -58,10 +71,12 @@ ECHO_DEV float gelu_tanh(float x) {
     return 0.5f * x * (1.f + tanhf(u));
 }
 
-// Tile order: bands of GROUP_N N-tiles; inside a band M is swept with the band's
-// N-tiles adjacent, so the CTAs in flight share a few A row blocks and one band
-// of W, which stay in L2 while the band is processed.
+// Tile order: bands of BAND_COLS columns; inside a band M is swept with the
+// band's N-tiles adjacent, so the CTAs in flight share a few A row blocks and one
+// band of W, which stay in L2 while the band is processed.
+template <int BN>
 ECHO_DEV void tile_coords(int t, int num_m, int num_n, int &mt, int &nt) {
+    constexpr int GROUP_N = Cfg<BN>::GROUP_N;
     const int band = t / (GROUP_N * num_m);
     const int first_n = band * GROUP_N;
     const int gn = min(GROUP_N, num_n - first_n);
@@ -70,86 +85,113 @@ ECHO_DEV void tile_coords(int t, int num_m, int num_n, int &mt, int &nt) {
     nt = first_n + r % gn;
 }
 
-// One accumulator row of a tile (thread = TMEM lane): tcgen05.ld 32 columns at a
-// time from `tacc`, bias, GELU, residual, store; EPI_ROWAMAX folds the row max.
-template <int EPI>
-ECHO_DEV void epilogue_row(const GemmParams &p, uint32_t tacc, int row, int n0) {
-    const bool row_ok = row < p.M;
-    int rrow = row;
-    if ((EPI & EPI_RES_BF16) && p.resid_rows && row_ok) rrow = p.resid_rows[row];
-    const int64_t orow = (p.out_rows && row_ok) ? p.out_rows[row] : row;
-    uint32_t rmax = 0;   // EPI_ROWAMAX: max |v| of this row's stored values, as bits
-    for (int c = 0; c < BN; c += 32) {
+// One warp's 32 rows x COLS columns of a tile, 32 columns at a time: tcgen05.ld
+// (a row per lane), through the warp's staging block (16-byte chunks XOR-swizzled
+// by the row, so that both sides spread over the banks), then 8 lanes per row
+// with 4 columns each: bias, GELU, residual and store run on whole row segments.
+// The residual is read before the accumulator is waited for.  `release` is called
+// once, as soon as the last of the accumulator has been read.
+template <int EPI, int COLS, typename Release>
+ECHO_DEV void epilogue_rows(const GemmParams &p, uint32_t tacc, uint8_t *stage, int row0, int n0,
+                            Release release) {
+    const int lane = threadIdx.x & 31, sub = lane >> 3, cc = lane & 7;
+    const bool lane_ok = row0 + lane < p.M;
+    int orow = row0 + lane, rrow = row0 + lane;   // of the warp's row `lane`
+    if (p.out_rows && lane_ok) orow = p.out_rows[row0 + lane];
+    if ((EPI & EPI_RES_BF16) && p.resid_rows && lane_ok) rrow = p.resid_rows[row0 + lane];
+    uint32_t rmax[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // EPI_ROWAMAX: max |v| of rows 4 i + sub, as bits
+    if (n0 >= p.N) release();
+#pragma unroll 1
+    for (int c = 0; c < COLS; c += 32) {
         const int col = n0 + c;
         if (col >= p.N) break;                       // warp-uniform
+        float4 rf[8];
+        uint2 rb[8];
+        if (EPI & EPI_RES_F32) {
+            const float *rp = static_cast<const float *>(p.resid) + col + 4 * cc;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int row = row0 + 4 * i + sub;
+                rf[i] = row < p.M ? __ldg(reinterpret_cast<const float4 *>(rp + (int64_t)row * p.N))
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
+        if (EPI & EPI_RES_BF16) {
+            const __nv_bfloat16 *rp = static_cast<const __nv_bfloat16 *>(p.resid) + col + 4 * cc;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int64_t rr = __shfl_sync(0xffffffffu, rrow, 4 * i + sub);
+                rb[i] = row0 + 4 * i + sub < p.M
+                            ? __ldg(reinterpret_cast<const uint2 *>(rp + rr * p.N)) : make_uint2(0, 0);
+            }
+        }
+        float bias[4] = {0.f, 0.f, 0.f, 0.f};
+        if (p.bias) {
+            const uint2 b = __ldg(reinterpret_cast<const uint2 *>(p.bias + col + 4 * cc));
+            bias[0] = bf16lo(b.x); bias[1] = bf16hi(b.x); bias[2] = bf16lo(b.y); bias[3] = bf16hi(b.y);
+        }
         uint32_t r[32];
         tmem_ld32(tacc + (uint32_t)c, r);
         tmem_ld_wait();
-        if (!row_ok) continue;
-        float v[32];
-        if (p.bias) {
-            const uint4 *bp = reinterpret_cast<const uint4 *>(p.bias + col);
+        if (c + 32 >= COLS || col + 32 >= p.N) release();
+        __syncwarp();                                // the previous block has been read
 #pragma unroll
-            for (int i = 0; i < 4; ++i) unpack8_bf16(__ldg(bp + i), v + 8 * i);
+        for (int k = 0; k < 8; ++k)
+            *reinterpret_cast<uint4 *>(stage + lane * 128 + ((k ^ (lane & 7)) * 16)) =
+                make_uint4(r[4 * k], r[4 * k + 1], r[4 * k + 2], r[4 * k + 3]);
+        __syncwarp();
 #pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] += __uint_as_float(r[i]);
-        } else {
+        for (int i = 0; i < 8; ++i) {
+            const int lr = 4 * i + sub;
+            const float4 a = *reinterpret_cast<const float4 *>(stage + lr * 128 + ((cc ^ (lr & 7)) * 16));
+            const int64_t o = __shfl_sync(0xffffffffu, orow, lr);
+            float v[4] = {a.x, a.y, a.z, a.w};
+            if (p.bias) {
 #pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-        }
-        if (EPI & EPI_GELU) {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = gelu_tanh(v[i]);
-        }
-        if (EPI & EPI_RES_BF16) {
-            const uint4 *rp = reinterpret_cast<const uint4 *>(
-                static_cast<const __nv_bfloat16 *>(p.resid) + (int64_t)rrow * p.N + col);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                float tt[8];
-                unpack8_bf16(__ldg(rp + i), tt);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) v[8 * i + e] += tt[e];
+                for (int e = 0; e < 4; ++e) v[e] += bias[e];
             }
-        }
-        if (EPI & EPI_RES_F32) {
-            const float4 *rp = reinterpret_cast<const float4 *>(
-                static_cast<const float *>(p.resid) + (int64_t)row * p.N + col);
+            if (EPI & EPI_GELU) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const float4 tt = __ldg(rp + i);
-                v[4 * i] += tt.x; v[4 * i + 1] += tt.y; v[4 * i + 2] += tt.z; v[4 * i + 3] += tt.w;
+                for (int e = 0; e < 4; ++e) v[e] = gelu_tanh(v[e]);
             }
-        }
-        if (EPI & EPI_OUT_F32) {
-            float4 *op = reinterpret_cast<float4 *>(static_cast<float *>(p.out) +
-                                                    orow * p.ldo + col);
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                op[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-        } else {
-            uint4 *op = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(p.out) +
-                                                  orow * p.ldo + col);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const uint4 pk = pack8_bf16(v + 8 * i);
-                op[i] = pk;
-                if (EPI & EPI_ROWAMAX) {
-                    const uint32_t w[4] = {pk.x, pk.y, pk.z, pk.w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        rmax = max(rmax, max((w[e] & 0x7FFFu) << 16, w[e] & 0x7FFF0000u));
-                }
+            if (EPI & EPI_RES_BF16) {
+                v[0] += bf16lo(rb[i].x); v[1] += bf16hi(rb[i].x);
+                v[2] += bf16lo(rb[i].y); v[3] += bf16hi(rb[i].y);
+            }
+            if (EPI & EPI_RES_F32) {
+                v[0] += rf[i].x; v[1] += rf[i].y; v[2] += rf[i].z; v[3] += rf[i].w;
+            }
+            if (row0 + lr >= p.M) continue;
+            if (EPI & EPI_OUT_F32) {
+                *reinterpret_cast<float4 *>(static_cast<float *>(p.out) + o * p.ldo + col + 4 * cc) =
+                    make_float4(v[0], v[1], v[2], v[3]);
+            } else {
+                const uint2 w = make_uint2(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]));
+                *reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(p.out) + o * p.ldo + col +
+                                           4 * cc) = w;
+                if (EPI & EPI_ROWAMAX)
+                    rmax[i] = max(rmax[i], max(max((w.x & 0x7FFFu) << 16, w.x & 0x7FFF0000u),
+                                               max((w.y & 0x7FFFu) << 16, w.y & 0x7FFF0000u)));
             }
         }
     }
-    if ((EPI & EPI_ROWAMAX) && row_ok) atomicMax(&p.row_amax[row], rmax);
+    if (EPI & EPI_ROWAMAX) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+#pragma unroll
+            for (int s = 1; s < 8; s *= 2)
+                rmax[i] = max(rmax[i], __shfl_xor_sync(0xffffffffu, rmax[i], s));
+            if (cc == 0 && row0 + 4 * i + sub < p.M) atomicMax(&p.row_amax[row0 + 4 * i + sub], rmax[i]);
+        }
+    }
 }
 
-template <int EPI>
+template <int EPI, int BN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
             const GemmParams p) {
+    using C = Cfg<BN>;
+    constexpr int STAGES = C::STAGES, STAGE_BYTES = C::STAGE_BYTES;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                 ~static_cast<uintptr_t>(1023));
@@ -172,7 +214,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], 8);   // lane 0 of the 4 epilogue warps of both CTAs
+            mbar_init(&acc_empty[b], 2 * EPI_WARPS);   // lane 0 of both CTAs' epilogue warps
         }
         mbar_init(&drain_bar, 1);
         abort_flag = 0;
@@ -181,7 +223,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         tma_prefetch_desc(&tmB);
     }
     cluster_sync_all();   // both CTAs' barriers exist before any arrival from the other CTA
-    if (warp == 2) tmem_alloc_pair(&tmem_slot, TMEM_COLS);
+    if (warp == 2) tmem_alloc_pair(&tmem_slot, C::TMEM_COLS);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -198,7 +240,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         bool ok = true;
         for (int t = pair; ok && t < num_tiles; t += num_pairs) {
             int mt, nt;
-            tile_coords(t, num_m, num_n, mt, nt);
+            tile_coords<BN>(t, num_m, num_n, mt, nt);
             for (int kb = 0; kb < num_kb; ++kb, ++it) {
                 const int s = it % STAGES;
                 if (!mbar_wait_cluster(&empty_bar[s], ((it / STAGES) & 1) ^ 1, abort_v, p.err)) {
@@ -259,7 +301,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 if (leader) {
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k)
-                        tc_mma_pair_f16(d_tmem, desc(a_lo + 2 * k), desc(b_lo + 2 * k), IDESC,
+                        tc_mma_pair_f16(d_tmem, desc(a_lo + 2 * k), desc(b_lo + 2 * k), C::IDESC,
                                         (kb | k) != 0);
                     tc_commit_pair(&empty_bar[s], 0x3);   // the stage is free in both CTAs
                 }
@@ -274,8 +316,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         }
     } else if (warp >= 4) {
         // ---------------- epilogue (both CTAs) ----------------
-        const int q = warp & 3;
+        // two warps per TMEM lane quarter, each with half of the columns
+        const int q = warp & 3, half = (warp - 4) >> 2;
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
+        uint8_t *stage = smem + STAGES * STAGE_BYTES + (warp - 4) * STG_BYTES;
         const uint32_t empty_even[2] = {mapa_shared(smem_u32(&acc_empty[0]), 0),
                                         mapa_shared(smem_u32(&acc_empty[1]), 0)};
         int local = 0;
@@ -286,12 +330,14 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             if (!ok) break;
             tc_fence_after();
             int mt, nt;
-            tile_coords(t, num_m, num_n, mt, nt);
-            epilogue_row<EPI>(p, tmem + lane_base + (uint32_t)(buf * BN),
-                              mt * 2 * BM + (int)rank * BM + q * 32 + lane, nt * BN);
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_remote(empty_even[buf]);
+            tile_coords<BN>(t, num_m, num_n, mt, nt);
+            epilogue_rows<EPI, BN / 2>(
+                p, tmem + lane_base + (uint32_t)(buf * BN + half * (BN / 2)), stage,
+                mt * 2 * BM + (int)rank * BM + q * 32, nt * BN + half * (BN / 2), [&]() {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_remote(empty_even[buf]);
+                });
         }
     }
     tc_fence_before();
@@ -299,7 +345,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     cluster_sync_all();   // neither CTA leaves while the other may still reach its memory
     if (warp == 2) {
         tc_fence_after();
-        tmem_dealloc_pair(tmem, TMEM_COLS);
+        tmem_dealloc_pair(tmem, C::TMEM_COLS);
     }
 }
 
@@ -315,13 +361,14 @@ int num_sms() {
     return cached[dev];
 }
 
-template <int EPI>
-echo_status run(const CUtensorMap &ta, const CUtensorMap &tb, const GemmParams &p, cudaStream_t st) {
+template <int EPI, int BN>
+echo_status run_bn(const CUtensorMap &ta, const CUtensorMap &tb, const GemmParams &p, cudaStream_t st) {
     static int pairs_max[64] = {};   // per device: co-resident CTA pairs (0: not set up yet)
+    constexpr int SMEM_BYTES = Cfg<BN>::SMEM_BYTES;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return ECHO_ERR_CUDA;
     if (!pairs_max[dev]) {   // a benign race computes the same value twice
-        if (cudaFuncSetAttribute(gemm_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(gemm_kernel<EPI, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  SMEM_BYTES) != cudaSuccess)
             return ECHO_ERR_CUDA;
         cudaLaunchConfig_t cfg = {};
@@ -329,15 +376,39 @@ echo_status run(const CUtensorMap &ta, const CUtensorMap &tb, const GemmParams &
         cfg.blockDim = dim3(THREADS, 1, 1);
         cfg.dynamicSmemBytes = SMEM_BYTES;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, gemm_kernel<EPI>, &cfg) != cudaSuccess || n < 1)
+        if (cudaOccupancyMaxActiveClusters(&n, gemm_kernel<EPI, BN>, &cfg) != cudaSuccess || n < 1)
             return ECHO_ERR_CUDA;
         pairs_max[dev] = n;
     }
     const int tiles = ((p.M + 2 * BM - 1) / (2 * BM)) * ((p.N + BN - 1) / BN);
     const int pairs = tiles < pairs_max[dev] ? tiles : pairs_max[dev];
     echo::LaunchScope ls(ECHO_K_GEMM, p.M, p.N, p.Kd, st);
-    gemm_kernel<EPI><<<2 * pairs, THREADS, SMEM_BYTES, st>>>(ta, tb, p);
+    gemm_kernel<EPI, BN><<<2 * pairs, THREADS, SMEM_BYTES, st>>>(ta, tb, p);
     return echo::last_launch_status();
+}
+
+// Tile width, by the cycles of the waves: a 64-deep k-block of 256 columns takes
+// 512 (the tensor rate), of 128 columns about 340 (the copies into shared memory),
+// plus about 600 a tile and the last tile's epilogue, which nothing overlaps.  128
+// columns spread a small output over more SM pairs: 1560 x 1024 x 1024 12.8 ->
+// 10.3 us, 1560 x 1024 x 4096 25.7 -> 21.4 us, 400 x 640 x 2048 16.8 -> 13.4 us,
+// 1563 x 4096 x 1024 25.5 -> 23.2 us; at 7800 x 1024 x 4096 they take 69 us
+// against 48, at 600 x 5120 x 5120 44 against 31, and the rule keeps 256.
+bool narrow_tiles(int M, int N, int Kd) {
+    const int64_t pairs = num_sms() / 2, nm = (M + 2 * BM - 1) / (2 * BM), kb = Kd / BK;
+    const int64_t w256 = (nm * ((N + 255) / 256) + pairs - 1) / pairs;
+    const int64_t w128 = (nm * ((N + 127) / 128) + pairs - 1) / pairs;
+    return w128 * (kb * 340 + 600) + 1500 < w256 * (kb * 512 + 600) + 3000;
+}
+
+template <int EPI>
+echo_status run(const echo::LinearArgs &a, const GemmParams &p, cudaStream_t st) {
+    const bool narrow = narrow_tiles(p.M, p.N, p.Kd);
+    CUtensorMap ta, tb;
+    if (!echo::make_tmap_bf16(&ta, a.A, (uint64_t)a.M, (uint64_t)a.Kd, (uint64_t)a.lda, BM) ||
+        !echo::make_tmap_bf16(&tb, a.W, (uint64_t)a.N, (uint64_t)a.Kd, (uint64_t)a.Kd, narrow ? 64 : 128))
+        return ECHO_ERR_CUDA;
+    return narrow ? run_bn<EPI, 128>(ta, tb, p, st) : run_bn<EPI, 256>(ta, tb, p, st);
 }
 
 }  // namespace
@@ -346,10 +417,6 @@ namespace echo {
 
 echo_status launch_linear(const LinearArgs &a, cudaStream_t st) {
     if (a.M <= 0) return ECHO_OK;
-    CUtensorMap ta, tb;
-    if (!make_tmap_bf16(&ta, a.A, (uint64_t)a.M, (uint64_t)a.Kd, (uint64_t)a.lda, BM) ||
-        !make_tmap_bf16(&tb, a.W, (uint64_t)a.N, (uint64_t)a.Kd, (uint64_t)a.Kd, BN / 2))
-        return ECHO_ERR_CUDA;
     GemmParams p;
     p.M = a.M; p.N = a.N; p.Kd = a.Kd;
     p.bias = static_cast<const __nv_bfloat16 *>(a.bias);
@@ -366,23 +433,23 @@ echo_status launch_linear(const LinearArgs &a, cudaStream_t st) {
     if (a.out_t == ECHO_F32) epi |= EPI_OUT_F32;
     if (a.row_amax) {
         if (epi != EPI_RES_F32) return ECHO_ERR_INVALID_ARG;   // bf16 out, fp32 residual only
-        return run<EPI_RES_F32 | EPI_ROWAMAX>(ta, tb, p, st);
+        return run<EPI_RES_F32 | EPI_ROWAMAX>(a, p, st);
     }
     switch (epi) {
-        case 0: return run<0>(ta, tb, p, st);
-        case EPI_GELU: return run<EPI_GELU>(ta, tb, p, st);
-        case EPI_RES_BF16: return run<EPI_RES_BF16>(ta, tb, p, st);
-        case EPI_RES_F32: return run<EPI_RES_F32>(ta, tb, p, st);
-        case EPI_GELU | EPI_RES_BF16: return run<EPI_GELU | EPI_RES_BF16>(ta, tb, p, st);
-        case EPI_GELU | EPI_RES_F32: return run<EPI_GELU | EPI_RES_F32>(ta, tb, p, st);
-        case EPI_OUT_F32: return run<EPI_OUT_F32>(ta, tb, p, st);
-        case EPI_GELU | EPI_OUT_F32: return run<EPI_GELU | EPI_OUT_F32>(ta, tb, p, st);
-        case EPI_RES_BF16 | EPI_OUT_F32: return run<EPI_RES_BF16 | EPI_OUT_F32>(ta, tb, p, st);
-        case EPI_RES_F32 | EPI_OUT_F32: return run<EPI_RES_F32 | EPI_OUT_F32>(ta, tb, p, st);
+        case 0: return run<0>(a, p, st);
+        case EPI_GELU: return run<EPI_GELU>(a, p, st);
+        case EPI_RES_BF16: return run<EPI_RES_BF16>(a, p, st);
+        case EPI_RES_F32: return run<EPI_RES_F32>(a, p, st);
+        case EPI_GELU | EPI_RES_BF16: return run<EPI_GELU | EPI_RES_BF16>(a, p, st);
+        case EPI_GELU | EPI_RES_F32: return run<EPI_GELU | EPI_RES_F32>(a, p, st);
+        case EPI_OUT_F32: return run<EPI_OUT_F32>(a, p, st);
+        case EPI_GELU | EPI_OUT_F32: return run<EPI_GELU | EPI_OUT_F32>(a, p, st);
+        case EPI_RES_BF16 | EPI_OUT_F32: return run<EPI_RES_BF16 | EPI_OUT_F32>(a, p, st);
+        case EPI_RES_F32 | EPI_OUT_F32: return run<EPI_RES_F32 | EPI_OUT_F32>(a, p, st);
         case EPI_GELU | EPI_RES_BF16 | EPI_OUT_F32:
-            return run<EPI_GELU | EPI_RES_BF16 | EPI_OUT_F32>(ta, tb, p, st);
+            return run<EPI_GELU | EPI_RES_BF16 | EPI_OUT_F32>(a, p, st);
         case EPI_GELU | EPI_RES_F32 | EPI_OUT_F32:
-            return run<EPI_GELU | EPI_RES_F32 | EPI_OUT_F32>(ta, tb, p, st);
+            return run<EPI_GELU | EPI_RES_F32 | EPI_OUT_F32>(a, p, st);
     }
     return ECHO_ERR_INVALID_ARG;
 }
