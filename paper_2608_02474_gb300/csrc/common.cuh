@@ -241,9 +241,12 @@ ECHO_DEV float4 ld_shared_cluster_f4(uint32_t cluster_addr) {
     return v;
 }
 
-// Arrive on an mbarrier given by its shared::cluster address (possibly another CTA's).
-ECHO_DEV void mbar_arrive_remote(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr)
+// Arrive on an mbarrier given by its shared::cluster address (possibly another
+// CTA's) without a release: it orders no earlier memory access, so the thread does
+// not wait for its global stores.  For handing back tensor memory whose loads have
+// completed (tcgen05.wait::ld, then tcgen05.fence::before_thread_sync).
+ECHO_DEV void mbar_arrive_remote_relaxed(uint32_t cluster_addr) {
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr)
                  : "memory");
 }
 
