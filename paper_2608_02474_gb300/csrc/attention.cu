@@ -190,6 +190,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
     volatile int *abort_v = &abort_flag;
+    pdl_enter();   // set up: from here on global memory is read and written
     // Register split (launch: 384 x 168 = 64512): the control warpgroup keeps
     // 48 per thread, the two softmax warpgroups take 224 (128*48 + 256*224 = 63488).
     if (warp < 4) {
@@ -589,6 +590,7 @@ attn_items_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
     volatile int *abort_v = &abort_flag;
+    pdl_enter();   // set up: from here on global memory is read and written
     // Register split as in the kernel above (launch: 384 x 168).
     if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 48;" ::: "memory");
@@ -964,7 +966,9 @@ echo_status launch_items(const void *Q, int64_t ldq, const void *K, const void *
     p.err = echo::device_error_ptr();
     const int grid = p.items < num_sms() ? p.items : num_sms();
     echo::LaunchScope ls(ECHO_K_ATTENTION, M, L, (int64_t)H * DH, st);
-    attn_items_kernel<DH, BN><<<grid, THREADS, C::SMEM, st>>>(tq, tk, tv, p);
+    echo::launch_chained(attn_items_kernel<DH, BN>, dim3(grid), dim3(THREADS), C::SMEM, st, tq,
+                         tk, tv,
+                         p);
     return echo::last_launch_status();
 }
 
@@ -1070,22 +1074,15 @@ echo_status launch_dh(const void *Q, int64_t ldq, const void *K, const void *V, 
     const int ntp = (M + TILES * BM - 1) / (TILES * BM);
     if (splits == 1) {
         echo::LaunchScope ls(ECHO_K_ATTENTION, M, L, (int64_t)H * DH, st);
-        attn_tc_kernel<DH, false><<<dim3(ntp, H), THREADS, Cfg<DH>::SMEM, st>>>(tq, tk, tv, p);
+        echo::launch_chained(attn_tc_kernel<DH, false>, dim3(ntp, H), dim3(THREADS),
+                             Cfg<DH>::SMEM, st,
+                             tq, tk, tv, p);
         return echo::last_launch_status();
     }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(ntp * splits), (unsigned)H, 1);
-    cfg.blockDim = dim3(THREADS, 1, 1);
-    cfg.dynamicSmemBytes = Cfg<DH>::SMEM;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)splits;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
     echo::LaunchScope ls(ECHO_K_ATTENTION, M, L, (int64_t)H * DH, st);
-    if (cudaLaunchKernelEx(&cfg, attn_tc_kernel<DH, true>, tq, tk, tv, p) != cudaSuccess)
+    if (echo::launch_chained_cluster((unsigned)splits, attn_tc_kernel<DH, true>,
+                                     dim3((unsigned)(ntp * splits), (unsigned)H), dim3(THREADS),
+                                     Cfg<DH>::SMEM, st, tq, tk, tv, p) != cudaSuccess)
         return ECHO_ERR_CUDA;
     return echo::last_launch_status();
 }

@@ -34,6 +34,7 @@ template <typename ST>
 __global__ void __launch_bounds__(kQuantThreads)
 quant_kernel(const ST *__restrict__ src, const int32_t *__restrict__ rows, int n_rows, int D,
              int8_t *__restrict__ q, float *__restrict__ scale, int *err) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int warps = blockDim.x >> 5;
     const int C = D >> 3;
@@ -115,6 +116,7 @@ template <typename DT>
 __global__ void __launch_bounds__(kVecThreads)
 dequant_kernel(const int8_t *__restrict__ q, const float *__restrict__ scale,
                const int32_t *__restrict__ rows, int n_rows, int D, DT *__restrict__ dst) {
+    pdl_enter();
     const int C = D >> 4;
     const int64_t total = (int64_t)n_rows * C;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
@@ -134,6 +136,7 @@ dequant_kernel(const int8_t *__restrict__ q, const float *__restrict__ scale,
 __global__ void rowmap_kernel(const int32_t *__restrict__ idx, int K, int NT,
                               int32_t *__restrict__ rowmap, uint32_t *__restrict__ zero,
                               int n_zero) {
+    pdl_enter();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n_zero) zero[i] = 0u;
     if (i >= NT) return;
@@ -152,6 +155,7 @@ __global__ void __launch_bounds__(kVecThreads)
 dequant_merge_kernel(const int8_t *__restrict__ q, const float *__restrict__ scale,
                      const int32_t *__restrict__ rowmap, const __nv_bfloat16 *__restrict__ y_act,
                      int NT, int D, __nv_bfloat16 *__restrict__ y) {
+    pdl_enter();
     const int C = D >> 4;
     const int64_t total = (int64_t)NT * C;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
@@ -187,6 +191,7 @@ __global__ void __launch_bounds__(kVecThreads)
 merge_quant_kernel(int8_t *__restrict__ q, float *__restrict__ scale,
                    const int32_t *__restrict__ rowmap, const uint32_t *__restrict__ amax_bits,
                    int NT, int D, __nv_bfloat16 *__restrict__ y, int *err) {
+    pdl_enter();
     const int C = D >> 4;
     const int64_t total = (int64_t)NT * C;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
@@ -254,10 +259,11 @@ void launch_quant(const void *src, echo_dtype st_t, const int32_t *rows, int32_t
     int *err = device_error_ptr();
     LaunchScope ls(ECHO_K_QUANT, n_rows, D, 0, st);
     if (st_t == ECHO_BF16)
-        quant_kernel<__nv_bfloat16><<<grid, kQuantThreads, 0, st>>>(
+        echo::launch_chained(quant_kernel<__nv_bfloat16>, dim3(grid), dim3(kQuantThreads), 0, st,
             static_cast<const __nv_bfloat16 *>(src), rows, n_rows, D, q, scale, err);
     else
-        quant_kernel<float><<<grid, kQuantThreads, 0, st>>>(static_cast<const float *>(src), rows,
+        echo::launch_chained(quant_kernel<float>, dim3(grid), dim3(kQuantThreads), 0, st,
+                             static_cast<const float *>(src), rows,
                                                             n_rows, D, q, scale, err);
 }
 
@@ -267,10 +273,11 @@ void launch_dequant(const int8_t *q, const float *scale, const int32_t *rows, in
     const int grid = grid_for((int64_t)n_rows * (D / 16), kVecThreads);
     LaunchScope ls(ECHO_K_DEQUANT, n_rows, D, 0, st);
     if (dt == ECHO_BF16)
-        dequant_kernel<__nv_bfloat16><<<grid, kVecThreads, 0, st>>>(
+        echo::launch_chained(dequant_kernel<__nv_bfloat16>, dim3(grid), dim3(kVecThreads), 0, st,
             q, scale, rows, n_rows, D, static_cast<__nv_bfloat16 *>(dst));
     else
-        dequant_kernel<float><<<grid, kVecThreads, 0, st>>>(q, scale, rows, n_rows, D,
+        echo::launch_chained(dequant_kernel<float>, dim3(grid), dim3(kVecThreads), 0, st, q,
+                             scale, rows, n_rows, D,
                                                             static_cast<float *>(dst));
 }
 
@@ -279,14 +286,15 @@ void launch_rowmap(const int32_t *idx, int32_t K, int32_t NT, int32_t *rowmap, u
     const int n = NT > n_zero ? NT : n_zero;
     if (n <= 0) return;
     LaunchScope ls(ECHO_K_ROWMAP, K, NT, 0, st);
-    rowmap_kernel<<<(n + 255) / 256, 256, 0, st>>>(idx, K, NT, rowmap, zero, n_zero);
+    echo::launch_chained(rowmap_kernel, dim3((n + 255) / 256), dim3(256), 0, st, idx, K, NT,
+                         rowmap, zero, n_zero);
 }
 
 void launch_dequant_merge(const int8_t *q, const float *scale, const int32_t *rowmap,
                           const void *y_act, int32_t NT, int32_t D, void *y, cudaStream_t st) {
     const int grid = grid_for((int64_t)NT * (D / 16), kVecThreads);
     LaunchScope ls(ECHO_K_MERGE, NT, D, 0, st);
-    dequant_merge_kernel<<<grid, kVecThreads, 0, st>>>(
+    echo::launch_chained(dequant_merge_kernel, dim3(grid), dim3(kVecThreads), 0, st,
         q, scale, rowmap, static_cast<const __nv_bfloat16 *>(y_act), NT, D,
         static_cast<__nv_bfloat16 *>(y));
 }
@@ -295,7 +303,8 @@ void launch_merge_quant(int8_t *q, float *scale, const int32_t *rowmap, const ui
                         int32_t NT, int32_t D, int32_t K, void *y, cudaStream_t st) {
     const int grid = grid_for((int64_t)NT * (D / 16), kVecThreads);
     LaunchScope ls(ECHO_K_MERGE_QUANT, NT, D, K, st);
-    merge_quant_kernel<<<grid, kVecThreads, 0, st>>>(q, scale, rowmap, amax, NT, D,
+    echo::launch_chained(merge_quant_kernel, dim3(grid), dim3(kVecThreads), 0, st, q, scale,
+                         rowmap, amax, NT, D,
                                                      static_cast<__nv_bfloat16 *>(y),
                                                      device_error_ptr());
 }

@@ -24,6 +24,7 @@ __global__ void __launch_bounds__(kGroup *kGroups)
 segment_energy_kernel(const float *__restrict__ audio, int seg_len, int n_fft, int log2n, int hop,
                       int n_frames, int n_bands, float *__restrict__ band_out,
                       float *__restrict__ seg_out) {
+    pdl_enter();
     extern __shared__ float2 sm[];
     const int half = n_fft >> 1;
     const int n_bins = half + 1;
@@ -162,6 +163,7 @@ template <int R>
 __global__ void __launch_bounds__(kWarpEnergyWarps * 32)
 segment_energy_warp_kernel(const float *__restrict__ audio, int seg_len, int hop, int n_frames,
                            int n_bands, float *__restrict__ band_out, float *__restrict__ seg_out) {
+    pdl_enter();
     constexpr int N = 32 * R, HALF = N / 2;
     constexpr int LOG2R = R == 2 ? 1 : R == 4 ? 2 : R == 8 ? 3 : 4;
     static_assert(R == 2 || R == 4 || R == 8 || R == 16, "R-point DFT in registers: R <= 16");
@@ -311,16 +313,20 @@ extern "C" echo_status echo_audio_energy(const float *audio, int64_t n_samples, 
         LaunchScope ls(ECHO_K_ENERGY, T, n_frames, n_fft, st);
         const int R = n_fft / 32;
         if (R == 2)
-            segment_energy_warp_kernel<2><<<T, kWarpEnergyWarps * 32, 0, st>>>(
+            echo::launch_chained(segment_energy_warp_kernel<2>, dim3(T),
+                                 dim3(kWarpEnergyWarps * 32), 0, st,
                 audio, seg_len, hop, n_frames, n_bands, band_energy, seg_energy);
         else if (R == 4)
-            segment_energy_warp_kernel<4><<<T, kWarpEnergyWarps * 32, 0, st>>>(
+            echo::launch_chained(segment_energy_warp_kernel<4>, dim3(T),
+                                 dim3(kWarpEnergyWarps * 32), 0, st,
                 audio, seg_len, hop, n_frames, n_bands, band_energy, seg_energy);
         else if (R == 8)
-            segment_energy_warp_kernel<8><<<T, kWarpEnergyWarps * 32, 0, st>>>(
+            echo::launch_chained(segment_energy_warp_kernel<8>, dim3(T),
+                                 dim3(kWarpEnergyWarps * 32), 0, st,
                 audio, seg_len, hop, n_frames, n_bands, band_energy, seg_energy);
         else
-            segment_energy_warp_kernel<16><<<T, kWarpEnergyWarps * 32, 0, st>>>(
+            echo::launch_chained(segment_energy_warp_kernel<16>, dim3(T),
+                                 dim3(kWarpEnergyWarps * 32), 0, st,
                 audio, seg_len, hop, n_frames, n_bands, band_energy, seg_energy);
         return last_launch_status();
     }
@@ -334,7 +340,7 @@ extern "C" echo_status echo_audio_energy(const float *audio, int64_t n_samples, 
         return ECHO_ERR_CUDA;
     {
         LaunchScope ls(ECHO_K_ENERGY, T, n_frames, n_fft, st);
-        segment_energy_kernel<<<T, kGroup * kGroups, smem, st>>>(
+        echo::launch_chained(segment_energy_kernel, dim3(T), dim3(kGroup * kGroups), smem, st,
             audio, seg_len, n_fft, log2n, hop, n_frames, n_bands, band_energy, seg_energy);
     }
     return last_launch_status();

@@ -279,6 +279,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
     volatile int *abort_v = &abort_flag;
+    pdl_enter();   // set up: from here on global memory is read and written
 
     if (warp == 0 && lane == 0) {
         // ---------------- TMA producer (both CTAs) ----------------
@@ -438,7 +439,8 @@ echo_status run_bn(const CUtensorMap &ta, const CUtensorMap &tb, const GemmParam
     const int tiles = ((p.M + 2 * BM - 1) / (2 * BM)) * ((p.N + BN - 1) / BN);
     const int pairs = tiles < pairs_max[dev] ? tiles : pairs_max[dev];
     echo::LaunchScope ls(ECHO_K_GEMM, p.M, p.N, p.Kd, st);
-    gemm_kernel<EPI, BN><<<2 * pairs, THREADS, SMEM_BYTES, st>>>(ta, tb, p);
+    echo::launch_chained(gemm_kernel<EPI, BN>, dim3(2 * pairs), dim3(THREADS), SMEM_BYTES, st,
+                         ta, tb, p);
     return echo::last_launch_status();
 }
 

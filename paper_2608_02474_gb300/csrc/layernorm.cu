@@ -51,6 +51,7 @@ template <typename T, int TPR>
 __global__ void __launch_bounds__(kThreads)
 layernorm_kernel(const T *__restrict__ in, const int32_t *__restrict__ rows, int n_rows, int D,
                  __nv_bfloat16 *__restrict__ out) {
+    pdl_enter();
     __shared__ float red[kThreads / 32];
     constexpr int RPB = kThreads / TPR;
     const int t = threadIdx.x % TPR;
@@ -113,6 +114,7 @@ template <int CPL>
 __global__ void __launch_bounds__(kThreads)
 layernorm_warp_bf16(const __nv_bfloat16 *__restrict__ in, const int32_t *__restrict__ rows,
                     int n_rows, int D, __nv_bfloat16 *__restrict__ out) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int warps = kThreads / 32;
     const int C = D >> 3;
@@ -195,6 +197,7 @@ layernorm_bulk_bf16(const __nv_bfloat16 *__restrict__ in, int n_rows, int D,
     if (threadIdx.x == 0) abort_flag = 0;
     fence_barrier_init();
     __syncthreads();
+    pdl_enter();
     volatile int *abort_v = &abort_flag;
     const int C = D >> 3;
     const float invD = 1.f / (float)D;
@@ -290,7 +293,8 @@ void launch_bulk_bf16(const __nv_bfloat16 *in, int n_rows, int D, __nv_bfloat16 
     }
     int grid = (n_rows + kBulkWarps - 1) / kBulkWarps;
     if (grid > 152 * 2) grid = 152 * 2;
-    layernorm_bulk_bf16<CPL><<<grid, kBulkWarps * 32, smem, st>>>(in, n_rows, D, out, scatter_map,
+    echo::launch_chained(layernorm_bulk_bf16<CPL>, dim3(grid), dim3(kBulkWarps * 32), smem, st,
+                         in, n_rows, D, out, scatter_map,
                                                                   out2, echo::device_error_ptr());
 }
 
@@ -300,7 +304,8 @@ void launch_warp_bf16(const __nv_bfloat16 *in, const int32_t *rows, int n_rows, 
     constexpr int RPB = kThreads / 32;
     int grid = (n_rows + RPB - 1) / RPB;
     if (grid > 152 * 8) grid = 152 * 8;
-    layernorm_warp_bf16<CPL><<<grid, kThreads, 0, st>>>(in, rows, n_rows, D, out);
+    echo::launch_chained(layernorm_warp_bf16<CPL>, dim3(grid), dim3(kThreads), 0, st, in, rows,
+                         n_rows, D, out);
 }
 
 // gathered rows of a bf16 input: the row packed in registers
@@ -323,6 +328,7 @@ constexpr int kRowThreads = 128, kRowChunks = 16;
 
 __global__ void __launch_bounds__(kRowThreads)
 layernorm_row_f32(const float *__restrict__ in, int D, __nv_bfloat16 *__restrict__ out) {
+    pdl_enter();
     __shared__ float red[2][kRowThreads / 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int C4 = D >> 2;
@@ -371,7 +377,7 @@ layernorm_row_f32(const float *__restrict__ in, int D, __nv_bfloat16 *__restrict
 // reject wider rows)
 void launch_all_f32(const float *in, int n_rows, int D, __nv_bfloat16 *out, cudaStream_t st) {
     if (n_rows <= 0) return;
-    layernorm_row_f32<<<n_rows, kRowThreads, 0, st>>>(in, D, out);
+    echo::launch_chained(layernorm_row_f32, dim3(n_rows), dim3(kRowThreads), 0, st, in, D, out);
 }
 
 // every row of a bf16 input, optionally also scattered through a map: the
@@ -400,12 +406,14 @@ void launch_t(const T *in, const int32_t *rows, int n_rows, int D, __nv_bfloat16
         constexpr int RPB = kThreads / 32;
         int grid = (n_rows + RPB - 1) / RPB;
         if (grid > 152 * 16) grid = 152 * 16;
-        layernorm_kernel<T, 32><<<grid, kThreads, 0, st>>>(in, rows, n_rows, D, out);
+        echo::launch_chained(layernorm_kernel<T, 32>, dim3(grid), dim3(kThreads), 0, st, in,
+                             rows, n_rows, D, out);
     } else {
         constexpr int RPB = kThreads / 128;
         int grid = (n_rows + RPB - 1) / RPB;
         if (grid > 152 * 16) grid = 152 * 16;
-        layernorm_kernel<T, 128><<<grid, kThreads, 0, st>>>(in, rows, n_rows, D, out);
+        echo::launch_chained(layernorm_kernel<T, 128>, dim3(grid), dim3(kThreads), 0, st, in,
+                             rows, n_rows, D, out);
     }
 }
 

@@ -48,6 +48,7 @@ ECHO_DEV bool bf16_nonfinite(uint32_t two) {
 __global__ void ref_release_kernel(const int32_t *__restrict__ rows, int n, int seg_len,
                                    const int32_t *__restrict__ ref, int32_t *refcount,
                                    int32_t *__restrict__ seg_lo, int32_t *__restrict__ seg_hi) {
+    pdl_enter();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < n) {
         const int i = rows[j];
@@ -107,6 +108,7 @@ __global__ void __launch_bounds__(kScanWarps * 32)
 ref_scan_kernel(const __nv_bfloat16 *__restrict__ src, const int32_t *__restrict__ seg_lo,
                 const int32_t *__restrict__ seg_hi, float tau, int D,
                 int32_t *__restrict__ src_pos) {
+    pdl_enter();
     extern __shared__ uint4 s_buf[];
     __shared__ float s_dot[kWin][kWin + 1];  // [w][t + 1], t = -1: the entering reference
     __shared__ float s_nv[kWin];
@@ -236,6 +238,7 @@ ECHO_DEV int block_scan(int v, int *warp_sums, int *total) {
 __global__ void __launch_bounds__(kAllocThreads)
 ref_alloc_kernel(const int32_t *__restrict__ src_pos, int n, const int32_t *__restrict__ refcount,
                  int R_cap, int32_t *__restrict__ free_list, int32_t *__restrict__ slot_of) {
+    pdl_enter();
     __shared__ int warp_sums[33];
     // rank the references in token order
     int run = 0;
@@ -272,6 +275,7 @@ ref_store_kernel(const __nv_bfloat16 *__restrict__ src, const int32_t *__restric
                  int D, const int32_t *__restrict__ src_pos, const int32_t *__restrict__ slot_of,
                  int8_t *__restrict__ q, float *__restrict__ scale, int32_t *__restrict__ ref,
                  int32_t *refcount, __nv_bfloat16 *__restrict__ pool, int *err) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int warps = blockDim.x >> 5;
     const int C = D >> 3;
@@ -396,6 +400,7 @@ template <int KIND>
 __global__ void __launch_bounds__(kVec)
 cache_read_kernel(echo_cache c, const int32_t *__restrict__ rows, int n,
                   __nv_bfloat16 *__restrict__ dst) {
+    pdl_enter();
     const int C = c.D >> 4;
     const int64_t total = (int64_t)n * C;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
@@ -415,6 +420,7 @@ template <int KIND>
 __global__ void __launch_bounds__(kVec)
 cache_merge_kernel(echo_cache c, const int32_t *__restrict__ rowmap,
                    const __nv_bfloat16 *__restrict__ y_act, __nv_bfloat16 *__restrict__ y) {
+    pdl_enter();
     const int C = c.D >> 4;
     const int64_t total = (int64_t)c.NT * C;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
@@ -439,6 +445,7 @@ cache_merge_kernel(echo_cache c, const int32_t *__restrict__ rowmap,
 __global__ void __launch_bounds__(kVec)
 cache_copy_kernel(const __nv_bfloat16 *__restrict__ src, const int32_t *__restrict__ rows, int n,
                   int D, __nv_bfloat16 *__restrict__ full, int *err) {
+    pdl_enter();
     const int C = D >> 3;
     const int64_t total = (int64_t)n * C;
     bool bad = false;
@@ -455,6 +462,7 @@ cache_copy_kernel(const __nv_bfloat16 *__restrict__ src, const int32_t *__restri
 
 __global__ void cache_stats_kernel(const int32_t *__restrict__ refcount, int R_cap,
                                    int32_t *__restrict__ out) {
+    pdl_enter();
     __shared__ int s_live, s_top;
     if (threadIdx.x == 0) {
         s_live = 0;
@@ -543,7 +551,8 @@ echo_status launch_cache_write(const echo_cache &c, const void *src, const int32
     }
     if (c.kind == ECHO_CACHE_BF16) {
         LaunchScope ls(ECHO_K_CACHE_COPY, n, c.D, 0, st);
-        cache_copy_kernel<<<grid_for((int64_t)n * (c.D / 8), kVec), kVec, 0, st>>>(
+        echo::launch_chained(cache_copy_kernel, dim3(grid_for((int64_t)n * (c.D / 8), kVec)),
+                             dim3(kVec), 0, st,
             s, rows, n, c.D, static_cast<__nv_bfloat16 *>(c.full), err);
         return last_launch_status();
     }
@@ -553,7 +562,7 @@ echo_status launch_cache_write(const echo_cache &c, const void *src, const int32
         return ECHO_ERR_CUDA;
     {
         LaunchScope ls(ECHO_K_REF_ALLOC, n, c.D, 0, st);
-        ref_release_kernel<<<(n + 255) / 256, 256, 0, st>>>(
+        echo::launch_chained(ref_release_kernel, dim3((n + 255) / 256), dim3(256), 0, st,
             rows, n, c.seg_len, c.ref, c.R_cap > 0 ? c.refcount : nullptr, w.seg_lo, w.seg_hi);
     }
     if (last_launch_status() != ECHO_OK) return ECHO_ERR_CUDA;
@@ -564,19 +573,22 @@ echo_status launch_cache_write(const echo_cache &c, const void *src, const int32
                                  (int)smem) != cudaSuccess)
             return ECHO_ERR_CUDA;
         LaunchScope ls(ECHO_K_REF_SCAN, n, c.D, 0, st);
-        ref_scan_kernel<<<nseg, kScanWarps * 32, smem, st>>>(s, w.seg_lo, w.seg_hi, c.tau, c.D,
+        echo::launch_chained(ref_scan_kernel, dim3(nseg), dim3(kScanWarps * 32), smem, st, s,
+                             w.seg_lo, w.seg_hi, c.tau, c.D,
                                                              w.src_pos);
     }
     if (last_launch_status() != ECHO_OK) return ECHO_ERR_CUDA;
     {
         LaunchScope ls(ECHO_K_REF_ALLOC, n, c.D, 0, st);
-        ref_alloc_kernel<<<1, kAllocThreads, 0, st>>>(w.src_pos, n, c.refcount, c.R_cap,
+        echo::launch_chained(ref_alloc_kernel, dim3(1), dim3(kAllocThreads), 0, st, w.src_pos, n,
+                             c.refcount, c.R_cap,
                                                        w.free_list, w.slot_of);
     }
     if (last_launch_status() != ECHO_OK) return ECHO_ERR_CUDA;
     {
         LaunchScope ls(ECHO_K_REF_STORE, n, c.D, 0, st);
-        ref_store_kernel<<<grid_for((int64_t)n * 32, kStoreThreads), kStoreThreads, 0, st>>>(
+        echo::launch_chained(ref_store_kernel, dim3(grid_for((int64_t)n * 32, kStoreThreads)),
+                             dim3(kStoreThreads), 0, st,
             s, rows, n, c.D, w.src_pos, w.slot_of, c.q, c.scale, c.ref, c.refcount,
             static_cast<__nv_bfloat16 *>(c.pool), err);
     }
@@ -594,9 +606,11 @@ void launch_cache_merge(const echo_cache &c, const int32_t *rowmap, const void *
     const __nv_bfloat16 *ya = static_cast<const __nv_bfloat16 *>(y_act);
     __nv_bfloat16 *yo = static_cast<__nv_bfloat16 *>(y);
     if (c.kind == ECHO_CACHE_BF16)
-        cache_merge_kernel<ECHO_CACHE_BF16><<<grid, kVec, 0, st>>>(c, rowmap, ya, yo);
+        echo::launch_chained(cache_merge_kernel<ECHO_CACHE_BF16>, dim3(grid), dim3(kVec), 0, st,
+                             c, rowmap, ya, yo);
     else
-        cache_merge_kernel<ECHO_CACHE_REF><<<grid, kVec, 0, st>>>(c, rowmap, ya, yo);
+        echo::launch_chained(cache_merge_kernel<ECHO_CACHE_REF>, dim3(grid), dim3(kVec), 0, st,
+                             c, rowmap, ya, yo);
 }
 
 }  // namespace echo
@@ -664,9 +678,11 @@ extern "C" echo_status echo_cache_read(const echo_cache *c, const int32_t *rows,
     LaunchScope ls(ECHO_K_DEQUANT, n_rows, c->D, 0, st);
     __nv_bfloat16 *d = static_cast<__nv_bfloat16 *>(dst);
     if (c->kind == ECHO_CACHE_BF16)
-        cache_read_kernel<ECHO_CACHE_BF16><<<grid, kVec, 0, st>>>(*c, rows, n_rows, d);
+        echo::launch_chained(cache_read_kernel<ECHO_CACHE_BF16>, dim3(grid), dim3(kVec), 0, st,
+                             *c, rows, n_rows, d);
     else
-        cache_read_kernel<ECHO_CACHE_REF><<<grid, kVec, 0, st>>>(*c, rows, n_rows, d);
+        echo::launch_chained(cache_read_kernel<ECHO_CACHE_REF>, dim3(grid), dim3(kVec), 0, st,
+                             *c, rows, n_rows, d);
     return last_launch_status();
 }
 
@@ -681,7 +697,8 @@ extern "C" echo_status echo_cache_stats(const echo_cache *c, int32_t *out, echo_
                                   ? ECHO_OK : ECHO_ERR_CUDA;
     {
         LaunchScope ls(ECHO_K_REF_ALLOC, c->R_cap, 0, 0, st);
-        cache_stats_kernel<<<1, 1024, 0, st>>>(c->refcount, c->R_cap, out);
+        echo::launch_chained(cache_stats_kernel, dim3(1), dim3(1024), 0, st, c->refcount,
+                             c->R_cap, out);
     }
     return last_launch_status();
 }

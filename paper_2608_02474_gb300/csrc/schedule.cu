@@ -75,6 +75,7 @@ template <typename T>
 __global__ void __launch_bounds__(kDeltaThreads, 4)
 step_delta_partial(const T *__restrict__ hp, const T *__restrict__ hc, int64_t n,
                    double *__restrict__ partial) {
+    pdl_enter();
     using C = Chunk<T>;
     constexpr int V = C::kVals;
     const int64_t chunks = n / V;
@@ -141,6 +142,7 @@ step_delta_partial(const T *__restrict__ hp, const T *__restrict__ hc, int64_t n
 
 __global__ void step_delta_final(const double *__restrict__ partial, int blocks, double xi,
                                  double *__restrict__ out, int *err) {
+    pdl_enter();
     double d = 0.0, c = 0.0;
     for (int j = threadIdx.x; j < blocks; j += 32) {
         d += partial[2 * j];
@@ -190,17 +192,19 @@ extern "C" echo_status echo_step_delta(const void *h_prev, const void *h_cur, ec
     {
         LaunchScope ls(ECHO_K_STEP_DELTA, n, ht == ECHO_BF16 ? 2 : 4, 0, st);
         if (ht == ECHO_BF16)
-            step_delta_partial<__nv_bfloat16><<<grid, kDeltaThreads, 0, st>>>(
+            echo::launch_chained(step_delta_partial<__nv_bfloat16>, dim3(grid),
+                                 dim3(kDeltaThreads), 0, st,
                 static_cast<const __nv_bfloat16 *>(h_prev), static_cast<const __nv_bfloat16 *>(h_cur),
                 n, partial);
         else
-            step_delta_partial<float><<<grid, kDeltaThreads, 0, st>>>(
+            echo::launch_chained(step_delta_partial<float>, dim3(grid), dim3(kDeltaThreads), 0, st,
                 static_cast<const float *>(h_prev), static_cast<const float *>(h_cur), n, partial);
     }
     if (last_launch_status() != ECHO_OK) return ECHO_ERR_CUDA;
     {
         LaunchScope ls(ECHO_K_STEP_DELTA, 0, 0, grid, st);
-        step_delta_final<<<1, 32, 0, st>>>(partial, grid, xi, out, device_error_ptr());
+        echo::launch_chained(step_delta_final, dim3(1), dim3(32), 0, st, partial, grid, xi, out,
+                             device_error_ptr());
     }
     return last_launch_status();
 }

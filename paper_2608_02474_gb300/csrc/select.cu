@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(kDriftThreads)
 drift_kernel(const XT *__restrict__ x, CacheView cv, const float *__restrict__ seg_energy, int T,
              int N, int NT, int D, float lam, float xi, int mode, float *__restrict__ scores,
              int *err) {
+    pdl_enter();
     __shared__ float s_emax;
     if (threadIdx.x < 32) {
         float m = 0.f;
@@ -299,6 +300,7 @@ ECHO_DEV void compact_in_index_order(KeyFn keys4, int n, int first, uint32_t thr
 __global__ void __launch_bounds__(kTopkThreads)
 topk_kernel(const float *__restrict__ scores, int NT, int K, int keys_in_smem,
             int32_t *__restrict__ idx) {
+    pdl_enter();
     extern __shared__ uint32_t skeys[];
     __shared__ int hist[2048];
     __shared__ int warp_sums[33];
@@ -396,6 +398,7 @@ ECHO_DEV int4 ld_shared_cluster_v4(uint32_t cluster_addr) {
 __global__ void __launch_bounds__(kTopkThreads)
 topk_cluster_kernel(const float *__restrict__ scores, int NT, int K, int slice,
                     int32_t *__restrict__ idx) {
+    pdl_enter();
     extern __shared__ uint4 skeys4[];
     __shared__ __align__(16) int hist[2048];                  // this CTA's counts
     __shared__ __align__(16) int red[3][kBinsPerRank];        // owned bins, one buffer a pass
@@ -537,27 +540,19 @@ echo_status launch_topk(const float *keys, int NT, int K, int32_t *idx, cudaStre
     if (!topk_smem_cap_raised()) return ECHO_ERR_CUDA;
     const int slice = ((NT + kTopkClusterCtas - 1) / kTopkClusterCtas + 3) & ~3;
     if (NT >= kTopkClusterMinKeys && slice <= kTopkSliceMax) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(kTopkClusterCtas, 1, 1);
-        cfg.blockDim = dim3(kTopkThreads, 1, 1);
-        cfg.dynamicSmemBytes = (size_t)slice * sizeof(uint32_t);
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = kTopkClusterCtas;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
         LaunchScope ls(ECHO_K_TOPK, NT, K, 0, st);
-        if (cudaLaunchKernelEx(&cfg, topk_cluster_kernel, keys, NT, K, slice, idx) != cudaSuccess)
+        if (launch_chained_cluster((unsigned)kTopkClusterCtas, topk_cluster_kernel,
+                                   dim3(kTopkClusterCtas), dim3(kTopkThreads),
+                                   (size_t)slice * sizeof(uint32_t), st, keys, NT, K, slice,
+                                   idx) != cudaSuccess)
             return ECHO_ERR_CUDA;
         return last_launch_status();
     }
     const size_t key_bytes = (size_t)NT * sizeof(uint32_t);
     const int in_smem = key_bytes <= (size_t)kTopkKeyBytesMax ? 1 : 0;
     LaunchScope ls(ECHO_K_TOPK, NT, K, 0, st);
-    topk_kernel<<<1, kTopkThreads, in_smem ? key_bytes : 0, st>>>(keys, NT, K, in_smem, idx);
+    echo::launch_chained(topk_kernel, dim3(1), dim3(kTopkThreads), in_smem ? key_bytes : 0, st,
+                         keys, NT, K, in_smem, idx);
     return last_launch_status();
 }
 
@@ -565,6 +560,7 @@ size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // idx[j] = floor(j NT / K): K evenly spaced tokens, ascending and distinct
 __global__ void uniform_kernel(int NT, int K, int32_t *__restrict__ idx) {
+    pdl_enter();
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < K; j += gridDim.x * blockDim.x)
         idx[j] = (int32_t)(((int64_t)j * NT) / K);
 }
@@ -615,11 +611,13 @@ extern "C" echo_status echo_select(const void *x, echo_dtype xt, const int8_t *c
     {
     LaunchScope ls(ECHO_K_DRIFT, NT, D, 0, st);
     if (xt == ECHO_BF16)
-        drift_kernel<__nv_bfloat16, kCacheInt8><<<grid, kDriftThreads, 0, st>>>(
+        echo::launch_chained(drift_kernel<__nv_bfloat16, kCacheInt8>, dim3(grid),
+                             dim3(kDriftThreads), 0, st,
             static_cast<const __nv_bfloat16 *>(x), CacheView{cache_q, cache_scale, nullptr, nullptr,
             nullptr}, seg_energy, T, N, NT, D, prm.lambda, prm.xi, prm.mode, sc, err);
     else
-        drift_kernel<float, kCacheInt8><<<grid, kDriftThreads, 0, st>>>(
+        echo::launch_chained(drift_kernel<float, kCacheInt8>, dim3(grid), dim3(kDriftThreads), 0,
+                             st,
             static_cast<const float *>(x), CacheView{cache_q, cache_scale, nullptr, nullptr,
             nullptr}, seg_energy, T, N, NT, D, prm.lambda, prm.xi, prm.mode, sc, err);
     }
@@ -694,11 +692,13 @@ extern "C" echo_status echo_select_static(const void *x, echo_dtype xt, const in
     {
         LaunchScope ls(ECHO_K_DRIFT, NT, D, 0, st);
         if (xt == ECHO_BF16)
-            drift_kernel<__nv_bfloat16, kCacheInt8><<<grid, kDriftThreads, 0, st>>>(
+            echo::launch_chained(drift_kernel<__nv_bfloat16, kCacheInt8>, dim3(grid),
+                                 dim3(kDriftThreads), 0, st,
                 static_cast<const __nv_bfloat16 *>(x), CacheView{cache_q, cache_scale, nullptr,
                 nullptr, nullptr}, seg_energy, T, N, NT, D, prm.lambda, prm.xi, prm.mode, sc, err);
         else
-            drift_kernel<float, kCacheInt8><<<grid, kDriftThreads, 0, st>>>(
+            echo::launch_chained(drift_kernel<float, kCacheInt8>, dim3(grid),
+                                 dim3(kDriftThreads), 0, st,
                 static_cast<const float *>(x), CacheView{cache_q, cache_scale, nullptr, nullptr,
                 nullptr}, seg_energy, T, N, NT, D, prm.lambda, prm.xi, prm.mode, sc, err);
     }
@@ -732,7 +732,7 @@ extern "C" echo_status echo_select_uniform(int32_t T, int32_t N, int32_t ratio_n
     const int grid = (K + 255) / 256;
     {
         LaunchScope ls(ECHO_K_UNIFORM, T * N, K, 0, st);
-        uniform_kernel<<<grid, 256, 0, st>>>(T * N, K, idx);
+        echo::launch_chained(uniform_kernel, dim3(grid), dim3(256), 0, st, T * N, K, idx);
     }
     return last_launch_status();
 }
@@ -798,17 +798,21 @@ extern "C" echo_status echo_select_cache(const void *x, echo_dtype xt, const ech
         const float *xf = static_cast<const float *>(x);
         if (c->kind == ECHO_CACHE_BF16) {
             if (bf)
-                drift_kernel<__nv_bfloat16, kCacheBf16><<<grid, kDriftThreads, 0, st>>>(
+                echo::launch_chained(drift_kernel<__nv_bfloat16, kCacheBf16>, dim3(grid),
+                                     dim3(kDriftThreads), 0, st,
                     xb, cv, seg_energy, T, N, NT, D, prm.lambda, prm.xi, prm.mode, sc, err);
             else
-                drift_kernel<float, kCacheBf16><<<grid, kDriftThreads, 0, st>>>(
+                echo::launch_chained(drift_kernel<float, kCacheBf16>, dim3(grid),
+                                     dim3(kDriftThreads), 0, st,
                     xf, cv, seg_energy, T, N, NT, D, prm.lambda, prm.xi, prm.mode, sc, err);
         } else {
             if (bf)
-                drift_kernel<__nv_bfloat16, kCacheRef><<<grid, kDriftThreads, 0, st>>>(
+                echo::launch_chained(drift_kernel<__nv_bfloat16, kCacheRef>, dim3(grid),
+                                     dim3(kDriftThreads), 0, st,
                     xb, cv, seg_energy, T, N, NT, D, prm.lambda, prm.xi, prm.mode, sc, err);
             else
-                drift_kernel<float, kCacheRef><<<grid, kDriftThreads, 0, st>>>(
+                echo::launch_chained(drift_kernel<float, kCacheRef>, dim3(grid),
+                                     dim3(kDriftThreads), 0, st,
                     xf, cv, seg_energy, T, N, NT, D, prm.lambda, prm.xi, prm.mode, sc, err);
         }
     }
