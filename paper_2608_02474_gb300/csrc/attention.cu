@@ -2,7 +2,8 @@
 // latents, keys and values over the complete latent set (self-attention) or the
 // audio condition tokens (cross-attention).
 //
-// Flash-style forward on the 5th-generation tensor cores.  One CTA per
+// Flash-style forward on the 5th-generation tensor cores, d = 128 (d = 64 has its
+// own variant below).  One CTA per
 // (two 128-query tiles, head), or a cluster of 2, 4 or 8 CTAs that split its key
 // blocks, 12 warps, with the two tiles in ping-pong so that one tile's softmax
 // runs while the tensor cores work on the other:
@@ -66,12 +67,12 @@ struct AttnParams {
 // The results of the CTAs of a cluster, each over its own key blocks, summed
 // through distributed shared memory: with the rows' maxima m_r and sums l_r of
 // every CTA, O = sum_r 2^(m_r - m) O_r / sum_r 2^(m_r - m) l_r, m = max_r m_r.
-// m_r and l_r go to the tile's finished Q buffer.  Each thread scales its row of
-// this CTA's O by 2^(m_own - m) / sum and stages it in fp32 over the ring (free:
+// m_r and l_r go to the tile's finished Q buffer.  Each thread scales its row (or
+// its half of one, HALVES 2) of this CTA's O by 2^(m_own - m) / sum and stages it in fp32 over the ring (free:
 // every MMA is done after the first barrier); then CTA r adds rows [256 r / S, 256 (r + 1) / S) of every CTA in
 // rank order, rounds and stores them.  Three cluster barriers, which the
 // control warps pass too; a CTA that gave up passes them without its results.
-template <int DH, int S>
+template <int DH, int WARPS, int S>
 ECHO_DEV void sum_split_rows(const AttnParams &p, uint32_t stage_addr, int split, int q0, int h) {
     constexpr int LPR = DH / 4;                 // lanes per row, one 16-byte chunk each
     constexpr int RPW = 32 / LPR;               // rows per warp-wide load
@@ -81,7 +82,7 @@ ECHO_DEV void sum_split_rows(const AttnParams &p, uint32_t stage_addr, int split
 #pragma unroll
     for (int r = 0; r < S; ++r) base[r] = mapa_shared(stage_addr, (uint32_t)r);
 #pragma unroll 2
-    for (int i = warp * RPW; i < ROWS; i += 8 * RPW) {
+    for (int i = warp * RPW; i < ROWS; i += WARPS * RPW) {
         const int row = split * ROWS + i + lane / LPR, cc = lane % LPR;
         const uint32_t off = (uint32_t)(row * DH * 4 + ((cc ^ (row & 7)) * 16));
         float4 v[S];
@@ -98,13 +99,13 @@ ECHO_DEV void sum_split_rows(const AttnParams &p, uint32_t stage_addr, int split
     }
 }
 
-template <int DH>
-ECHO_DEV void combine_splits(const AttnParams &p, uint8_t *stage, float2 *own_ml, uint32_t o_tmem,
-                             int row, float m_own, float l_own, bool ok, int splits, int split,
+template <int DH, int HALVES>
+ECHO_DEV void combine_splits(const AttnParams &p, uint8_t *stage, float2 *own_ml, int half,
+                             uint32_t o_tmem, int row, float m_own, float l_own, bool ok, int splits, int split,
                              int q0, int h) {
     static_assert(TILES * BM * DH * 4 <= Cfg<DH>::RING * Cfg<DH>::SLOT_BYTES, "staged over the ring");
     if (l_own == 0.f) m_own = -INFINITY;
-    *own_ml = make_float2(m_own, l_own);
+    if (half == 0) *own_ml = make_float2(m_own, l_own);
     __syncwarp();
     cluster_sync_all();
     const uint32_t ml_addr = smem_u32(own_ml);
@@ -119,7 +120,8 @@ ECHO_DEV void combine_splits(const AttnParams &p, uint8_t *stage, float2 *own_ml
     const float f = ex2_approx(m_own - m) / l;
     if (ok) {   // warp-uniform
 #pragma unroll
-        for (int c = 0; c < DH / 32; ++c) {
+        for (int hc = 0; hc < DH / 32 / HALVES; ++hc) {
+            const int c = half * (DH / 32 / HALVES) + hc;
             uint32_t o[32];
             tmem_ld32(o_tmem + 32 * c, o);
             tmem_ld_wait();
@@ -133,9 +135,9 @@ ECHO_DEV void combine_splits(const AttnParams &p, uint8_t *stage, float2 *own_ml
     __syncwarp();
     cluster_sync_all();
     const uint32_t stage_addr = smem_u32(stage);
-    if (splits == 2) sum_split_rows<DH, 2>(p, stage_addr, split, q0, h);
-    else if (splits == 4) sum_split_rows<DH, 4>(p, stage_addr, split, q0, h);
-    else sum_split_rows<DH, 8>(p, stage_addr, split, q0, h);
+    if (splits == 2) sum_split_rows<DH, 8 * HALVES, 2>(p, stage_addr, split, q0, h);
+    else if (splits == 4) sum_split_rows<DH, 8 * HALVES, 4>(p, stage_addr, split, q0, h);
+    else sum_split_rows<DH, 8 * HALVES, 8>(p, stage_addr, split, q0, h);
     __syncwarp();
     cluster_sync_all();   // no CTA leaves while another may still read its rows
 }
@@ -447,10 +449,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         if (ok) tc_fence_after();
         if constexpr (SPLIT) {
             // the rows' maxima and sums in the tile's Q, the scaled rows over the ring
-            combine_splits<DH>(p, Ring,
-                               reinterpret_cast<float2 *>(Qs + t * C::Q_BYTES) + quad * 32 + lane,
-                               tmem + lane_base + o_col, t * BM + quad * 32 + lane, m_used, l, ok,
-                               splits, split, q0, h);
+            combine_splits<DH, 1>(p, Ring,
+                                  reinterpret_cast<float2 *>(Qs + t * C::Q_BYTES) + quad * 32 + lane, 0,
+                                  tmem + lane_base + o_col, t * BM + quad * 32 + lane, m_used, l, ok,
+                                  splits, split, q0, h);
         } else if (ok) {
             const float inv = 1.f / l;
             // The warp's 32 rows of O go through its quarter of Q_t (free now:
@@ -481,6 +483,387 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 #pragma unroll
             for (int k = 0; k < 32 / RPI; ++k) {
                 const int rr = k * RPI + lane / CH, cc = lane % CH;
+                const uint4 v =
+                    *reinterpret_cast<const uint4 *>(stage + rr * RB + ((cc ^ (rr & (CH - 1))) * 16));
+                const int grow = q0 + t * BM + quad * 32 + rr;
+                if (grow < p.M)
+                    *reinterpret_cast<uint4 *>(p.O + (int64_t)grow * p.ldo + h * DH + 8 * cc) = v;
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 2) {
+        tc_fence_after();
+        tmem_dealloc(tmem, TMEM_COLS);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Head size 64: the same roles, with two changes.  O takes only 2 x 64 columns, so
+// tensor memory holds three S buffers (0, 128, 256; O at 384): the next block's S
+// of a tile is computed while its softmax still works on this block's, instead of
+// after the P V that follows it.  And 16 softmax warps, two per 32 rows with 64
+// keys each.  The halves of a row agree on its maximum (first block) and on a redo
+// at one 64-thread barrier per block, and add up their sums at the end.  K_j and
+// V_j share a ring slot: one wait a block less on the issuing warp, which bounds
+// the kernel (24 MMAs of 32 to 64 cycles a block, and about 130 cycles a wait).
+// 16 heads, against the layout of attn_tc_kernel: 7800 x 7800 312 -> 243 us (305
+// with 16 softmax warps alone, 276 with the third S buffer, 243 with the shared
+// slot), 1560 x 7800 77 -> 62 us.  At d = 128 16 softmax warps gained nothing.
+// ---------------------------------------------------------------------------
+constexpr int D64_THREADS = 640;      // 4 control warps + 4 softmax warpgroups
+constexpr int S_BUFS = 3;
+constexpr uint32_t D64_O_COL = S_BUFS * BN;
+constexpr int D64_PAIRS = 5;          // ring of key blocks, K_j and V_j under one barrier
+constexpr int D64_SMEM = TILES * Cfg<64>::Q_BYTES + D64_PAIRS * 2 * Cfg<64>::SLOT_BYTES +
+                         TILES * 2 * BM * 4 + 1024;   // and the exchange of a row's halves
+
+template <bool SPLIT>
+__global__ void __launch_bounds__(D64_THREADS, 1)
+attn_d64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
+    using C = Cfg<64>;
+    constexpr int DH = 64;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                                ~static_cast<uintptr_t>(1023));
+    constexpr int RING = D64_PAIRS, PAIR_BYTES = 2 * C::SLOT_BYTES;
+    uint8_t *Qs = smem;                                  // [TILES][Q_BYTES]
+    uint8_t *Ring = Qs + TILES * C::Q_BYTES;             // [RING][K_j, V_j]
+    // a row's value of either half of its keys, for the other half (max, sum, redo)
+    float(*row_x)[2][BM] = reinterpret_cast<float(*)[2][BM]>(Ring + RING * PAIR_BYTES);
+
+    // Every barrier is reused only after its previous phase has been observed
+    // by its waiter, so no waiter can fall two phases behind.
+    __shared__ __align__(8) uint64_t q_full, ring_full[RING_MAX], ring_empty[RING_MAX];
+    __shared__ __align__(8) uint64_t s_full[S_BUFS], p_full[S_BUFS], pv_done[TILES];
+    __shared__ __align__(8) uint64_t drain;
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int h = blockIdx.y;
+    // the CTAs of a cluster share the queries and split the key blocks
+    const int splits = SPLIT ? (int)cluster_nctarank() : 1, split = SPLIT ? (int)cluster_ctarank() : 0;
+    const int q0 = ((int)blockIdx.x / splits) * (TILES * BM);
+    const int nb_all = (p.L + BN - 1) / BN;
+    const int kb0 = SPLIT ? (int)((int64_t)nb_all * split / splits) : 0;   // this CTA's first block
+    const int nb = SPLIT ? (int)((int64_t)nb_all * (split + 1) / splits) - kb0 : nb_all;
+
+    if (threadIdx.x == 0) {
+        mbar_init(&q_full, 1);
+        for (int i = 0; i < RING; ++i) { mbar_init(&ring_full[i], 1); mbar_init(&ring_empty[i], 1); }
+        for (int b = 0; b < S_BUFS; ++b) {
+            mbar_init(&s_full[b], 1);
+            mbar_init(&p_full[b], 8);    // one arrival per softmax warp of the tile
+        }
+        for (int t = 0; t < TILES; ++t) mbar_init(&pv_done[t], 1);
+        mbar_init(&drain, 1);
+        abort_flag = 0;
+        fence_barrier_init();
+        tma_prefetch_desc(&tmQ);
+        tma_prefetch_desc(&tmK);
+        tma_prefetch_desc(&tmV);
+    }
+    if (warp == 2) tmem_alloc(&tmem_slot, TMEM_COLS);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+    volatile int *abort_v = &abort_flag;
+    pdl_enter();   // set up: from here on global memory is read and written
+    // Register split (launch: 640 x 96 = 61440): the control warpgroup keeps 56 per
+    // thread, the four softmax warpgroups take 104 (128*56 + 512*104 = 60416).
+    if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 56;" ::: "memory");
+    if (warp == 0 && lane == 0) {
+        // ---------------- TMA producer: Q0, Q1, then K_0, V_0, K_1, V_1, ... ----------------
+        const int x0 = h * DH;
+        mbar_arrive_expect_tx(&q_full, TILES * C::Q_BYTES);
+        for (int t = 0; t < TILES; ++t)
+            for (int a = 0; a < C::ATOMS; ++a)
+                tma_load_2d(Qs + t * C::Q_BYTES + a * ATOM_BYTES, &tmQ, &q_full, x0 + 64 * a,
+                            q0 + t * BM);
+        int issued = 0;
+        for (int j = 0; j < nb; ++j) {
+            const int slot = j % RING;
+            if (!mbar_wait(&ring_empty[slot], ((j / RING) & 1) ^ 1, abort_v, p.err)) break;
+            mbar_arrive_expect_tx(&ring_full[slot], PAIR_BYTES);
+            uint8_t *dst = Ring + slot * PAIR_BYTES;
+            tma_load_2d(dst, &tmK, &ring_full[slot], x0, (kb0 + j) * BN);
+            tma_load_2d(dst + C::SLOT_BYTES, &tmV, &ring_full[slot], x0, (kb0 + j) * BN);
+            issued = j + 1;
+        }
+        if (*abort_v) {  // let this CTA's copies land before it exits
+            mbar_wait(&q_full, 0, abort_v, nullptr, 100000000ull);
+            for (int j = issued - RING < 0 ? 0 : issued - RING; j < issued; ++j)
+                mbar_wait(&ring_full[j % RING], (j / RING) & 1, abort_v, nullptr, 100000000ull);
+        }
+    } else if (warp == 1) {
+        // ---------------- MMA issuer ----------------
+        // Work items k = 2 j + t (key block j, tile t) in S buffer k mod 3.  Order:
+        //   S(0) S(1) S(2) | PV(0) S(3) | PV(1) S(4) | PV(2) S(5) | ...
+        // S(k + 3) goes over P(k) right after P V of item k has been issued (MMAs of
+        // one thread run in order), and S(k + 2), the tile's next block, is done
+        // while its softmax still works on item k.  The whole warp runs the loop,
+        // one elected lane issues, as in attn_tc_kernel.  Barriers are per buffer:
+        // item k + 3 cannot reach one before item k has been seen on it.
+        const bool leader = elect_one_sync();
+        // Shared-memory descriptors as two words: the low word holds the start
+        // address in 16-byte units and the leading byte offset, the high word the
+        // 1024-byte stride of eight 128-byte rows, the descriptor version and the
+        // 128-byte swizzle.  A K step only adds a constant to the low word.
+        constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
+        constexpr uint32_t LO_K = 1u << 16;                            // K-major: LBO unused
+        constexpr uint32_t LO_MN = (uint32_t)(ATOM_BYTES >> 4) << 16;  // MN-major: LBO = one atom
+        const uint32_t q_lo = ((smem_u32(Qs) & 0x3FFFFu) >> 4) | LO_K;
+        const uint32_t ring_lo = (smem_u32(Ring) & 0x3FFFFu) >> 4;
+        auto desc = [](uint32_t lo) -> uint64_t { return ((uint64_t)DESC_HI << 32) | lo; };
+        auto wait_all = [&](uint64_t *bar, uint32_t parity) -> bool {
+            return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_v, p.err));
+        };
+        bool ok = wait_all(&q_full, 0);
+        auto mma_s = [&](int t, int buf, int slot) {
+            const uint32_t a_lo = q_lo + (uint32_t)t * (C::Q_BYTES >> 4);
+            const uint32_t b_lo = (ring_lo + (uint32_t)slot * (PAIR_BYTES >> 4)) | LO_K;
+            const uint32_t d = tmem + (uint32_t)(buf * BN);
+#pragma unroll
+            for (int kk = 0; kk < DH / 16; ++kk)
+                tc_mma_f16(d, desc(a_lo + 2 * kk), desc(b_lo + 2 * kk), C::IDESC_S, kk > 0);
+        };
+        auto mma_pv = [&](int t, int buf, int slot, uint32_t acc0) {
+            const uint32_t b_lo =
+                (ring_lo + (uint32_t)slot * (PAIR_BYTES >> 4) + (C::SLOT_BYTES >> 4)) | LO_MN;
+            const uint32_t d = tmem + D64_O_COL + (uint32_t)(t * DH);
+            const uint32_t a = tmem + (uint32_t)(buf * BN);
+            tc_mma_f16_tmem_a(d, a, desc(b_lo), C::IDESC_PV, acc0);
+#pragma unroll
+            for (int kk = 1; kk < BN / 16; ++kk)
+                tc_mma_f16_tmem_a(d, a + 8 * kk, desc(b_lo + (uint32_t)(kk * 2048 >> 4)), C::IDESC_PV, 1u);
+        };
+        const int items = 2 * nb;
+        // ring slots of the next S's and the next P V's key block; S comes first and
+        // waits for both halves of the pair, P V releases it
+        int ks = 0, vs = 0;
+        uint32_t kph = 0;
+        auto issue_s = [&](int k, int buf) -> bool {
+            if (!(k & 1)) {                                      // first use of this key block
+                if (!wait_all(&ring_full[ks], kph)) return false;
+                tc_fence_after();
+            }
+            if (leader) {
+                mma_s(k & 1, buf, ks);
+                tc_commit(&s_full[buf]);
+            }
+            __syncwarp();
+            if ((k & 1) && ++ks == RING) { ks = 0; kph ^= 1u; }
+            return true;
+        };
+        for (int k = 0; ok && k < 3 && k < items; ++k) ok = issue_s(k, k);
+        int buf = 0;
+        uint32_t pph = 0;
+        for (int k = 0; ok && k < items; ++k) {
+            if (!wait_all(&p_full[buf], pph)) { ok = false; break; }
+            tc_fence_after();
+            if (leader) {
+                mma_pv(k & 1, buf, vs, k > 1 ? 1u : 0u);
+                tc_commit(&pv_done[k & 1]);
+                if (k & 1) tc_commit(&ring_empty[vs]);           // K_j and V_j no longer needed
+            }
+            __syncwarp();
+            if ((k & 1) && ++vs == RING) vs = 0;
+            if (k + 3 < items) ok = issue_s(k + 3, buf);
+            if (++buf == S_BUFS) { buf = 0; pph ^= 1u; }
+        }
+        if (!ok && leader) {  // wait for the MMAs already issued before tensor memory is freed
+            tc_commit(&drain);
+            mbar_wait(&drain, 0, abort_v, nullptr, 100000000ull);
+        }
+    }
+    if constexpr (SPLIT) {   // the three cluster barriers of combine_splits
+        __syncwarp();
+        cluster_sync_all();
+        cluster_sync_all();
+        cluster_sync_all();
+    }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 104;" ::: "memory");
+        // ------- softmax / correction / epilogue: half the keys of tile t's rows -------
+        const int t = (warp - 4) >> 3, half = ((warp - 4) >> 2) & 1;
+        const int quad = warp & 3;
+        const int row = quad * 32 + lane;                    // of the tile
+        const int bar_id = 1 + t * 4 + quad;                 // the two warps of these 32 rows
+        const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
+        const uint32_t o_col = D64_O_COL + (uint32_t)(t * DH);
+        const float sl2 = p.scale_log2;
+        constexpr int HN = BN / 2, HD = DH / 2;              // keys and O columns of one half
+        float m_used = -INFINITY, l = 0.f;
+        bool ok = true;
+        int buf = t;                                         // S buffer of item 2 j + t
+        uint32_t sph = 0;
+        for (int j = 0; j < nb; ++j) {
+            const uint32_t s_col = (uint32_t)(buf * BN);
+            // a wait that gave up is told to the other half at the vote below, so that
+            // both warps of the rows leave the loop at the same block
+            ok = __all_sync(0xffffffffu, mbar_wait(&s_full[buf], sph, abort_v, p.err));
+            tc_fence_after();
+            const int kvalid = p.L - (kb0 + j) * BN - half * HN;   // keys of this half that exist
+            float sv[HN];
+            auto load_s = [&]() {
+#pragma unroll
+                for (int c = 0; c < HN / 32; ++c)
+                    tmem_ld32(tmem + lane_base + s_col + half * HN + 32 * c,
+                              reinterpret_cast<uint32_t *>(sv + 32 * c));
+                tmem_ld_wait();
+                if (kvalid < HN) {                           // tail block only
+#pragma unroll
+                    for (int i = 0; i < HN; ++i)
+                        if (i >= kvalid) sv[i] = -INFINITY;
+                }
+            };
+            load_s();
+            // The running max m_used is taken from the first block only.  Later
+            // blocks form P with it directly: the result is exact after the final
+            // division by the row sum, and fp32 / bf16 keep their precision at any
+            // exponent, so a rescale is needed only when P could overflow.  A half
+            // block's row sum bounds its largest P; when it exceeds 2^64 (or is
+            // not finite) the block is redone with a fresh max and O, l rescaled.
+            auto half_max = [&]() -> float {
+                float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                for (int i = 0; i < HN; i += 8) {
+                    m4[0] = fmax3(m4[0], sv[i], sv[i + 1]);
+                    m4[1] = fmax3(m4[1], sv[i + 2], sv[i + 3]);
+                    m4[2] = fmax3(m4[2], sv[i + 4], sv[i + 5]);
+                    m4[3] = fmax3(m4[3], sv[i + 6], sv[i + 7]);
+                }
+                return fmaxf(fmax3(m4[0], m4[1], m4[2]), m4[3]);
+            };
+            // the larger of this half's and the other half's value for the row
+            auto row_max = [&](float v) -> float {
+                row_x[t][half][row] = v;
+                named_bar_sync(bar_id, 64);
+                return fmaxf(v, row_x[t][half ^ 1][row]);
+            };
+            // P = 2^(s*scale - m) on fp32 pairs, rounded to bf16 pairs; returns
+            // the row sum of this half block
+            uint32_t pk[HN / 2];
+            auto exp_pass = [&]() -> float {
+                const uint64_t scale2 = f2_pack(sl2, sl2);
+                const uint64_t negm2 = f2_pack(-m_used, -m_used);
+                uint64_t acc2[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+                for (int i = 0; i < HN / 2; ++i) {
+                    float x0, x1;
+                    f2_unpack(f2_fma(f2_pack(sv[2 * i], sv[2 * i + 1]), scale2, negm2), x0, x1);
+                    const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
+                    pk[i] = pack_bf16(p0, p1);
+                    acc2[i & 3] = f2_add(acc2[i & 3], f2_pack(p0, p1));
+                }
+                float a0, a1;
+                f2_unpack(f2_add(f2_add(acc2[0], acc2[1]), f2_add(acc2[2], acc2[3])), a0, a1);
+                return a0 + a1;
+            };
+            if (j == 0) {
+                m_used = row_max(half_max()) * sl2;
+                // a CTA whose first keys all score -inf adds nothing to the sums
+                // of the others instead of NaN
+                if (SPLIT && m_used == -INFINITY) m_used = 0.f;
+            }
+            float bsum = exp_pass();
+            const bool redo = !(bsum <= 1.8446744e19f);     // > 2^64, inf or NaN
+            // P goes over the first 64 columns of S_t, which half 0 has read by
+            // then: both warps of the rows meet here, and agree on a redo
+            tc_fence_before();
+            const bool any_redo = named_bar_or(bar_id, 64, redo || !ok);
+            tc_fence_after();
+            if (any_redo) {                                   // rare: both warps take it
+                ok = !named_bar_or(bar_id, 64, !ok);
+                if (!ok) break;
+                load_s();
+                const float m_blk = row_max(half_max());
+                named_bar_sync(bar_id, 64);                  // both have read the maxima
+                const float row_redo = row_max(redo ? 1.f : 0.f);
+                float alpha = 1.f;
+                if (row_redo != 0.f) {
+                    const float m_new = fmaxf(m_used, m_blk * sl2);
+                    alpha = ex2_approx(m_used - m_new);
+                    l *= alpha;
+                    m_used = m_new;
+                }
+                if (j > 0) {   // O_t is settled once P V of the block before is done
+                    mbar_wait(&pv_done[t], (j - 1) & 1, abort_v, p.err);
+                    __syncwarp();
+                    tc_fence_after();
+#pragma unroll
+                    for (int c = 0; c < HD / 32; ++c) {
+                        uint32_t o[32];
+                        tmem_ld32(tmem + lane_base + o_col + half * HD + 32 * c, o);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int i = 0; i < 32; ++i)
+                            o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                        tmem_st32(tmem + lane_base + o_col + half * HD + 32 * c, o);
+                    }
+                    tmem_st_wait();
+                }
+                load_s();                                     // S again: the max took its registers
+                tc_fence_before();
+                named_bar_sync(bar_id, 64);                   // before either stores its P
+                tc_fence_after();
+                bsum = exp_pass();
+            }
+            l += bsum;
+            // P into TMEM columns [0, 64) of S_t, half 0 first
+            tmem_st32(tmem + lane_base + s_col + half * (HN / 2), pk);
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&p_full[buf]);
+            if ((buf += 2) >= S_BUFS) { buf -= S_BUFS; sph ^= 1u; }
+        }
+        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&pv_done[t], (nb - 1) & 1, abort_v, p.err));
+        if (ok) tc_fence_after();
+        ok = !named_bar_or(bar_id, 64, !ok);                 // both warps of the rows, or neither
+        row_x[t][half][row] = l;                             // the row's sum over both halves
+        named_bar_sync(bar_id, 64);
+        l = row_x[t][0][row] + row_x[t][1][row];
+        if constexpr (SPLIT) {
+            // the rows' maxima and sums in the tile's Q, the scaled rows over the ring
+            combine_splits<DH, 2>(p, Ring, reinterpret_cast<float2 *>(Qs + t * C::Q_BYTES) + row, half,
+                               tmem + lane_base + o_col, t * BM + row, m_used, l, ok, splits, split,
+                               q0, h);
+        } else if (ok) {
+            const float inv = 1.f / l;
+            // The 32 rows of O go through their quarter of Q_t (free now: every
+            // MMA that read Q_t is done), half the columns from each warp, and
+            // leave in whole row segments, CH lanes per row, half the rows by each
+            // warp.  The 16-byte chunks of a staged row are XOR-swizzled by the row
+            // so that both the row-per-lane writes and the chunk-per-lane reads
+            // spread over the shared-memory banks.
+            constexpr int RB = DH * 2, CH = RB / 16;          // bytes and 16-byte chunks per row
+            uint8_t *stage = Qs + t * C::Q_BYTES + quad * 32 * RB;
+#pragma unroll
+            for (int c = 0; c < HD / 32; ++c) {
+                uint32_t o[32];
+                tmem_ld32(tmem + lane_base + o_col + half * HD + 32 * c, o);
+                tmem_ld_wait();
+                float f[32];
+#pragma unroll
+                for (int i = 0; i < 32; ++i) f[i] = __uint_as_float(o[i]) * inv;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int cc = half * (CH / 2) + 4 * c + i;
+                    *reinterpret_cast<uint4 *>(stage + lane * RB + ((cc ^ (lane & (CH - 1))) * 16)) =
+                        pack8_bf16(f + 8 * i);
+                }
+            }
+            named_bar_sync(bar_id, 64);
+            constexpr int RPI = 32 / CH;                        // rows per warp-wide store
+#pragma unroll
+            for (int k = 0; k < 16 / RPI; ++k) {
+                const int rr = half * 16 + k * RPI + lane / CH, cc = lane % CH;
                 const uint4 v =
                     *reinterpret_cast<const uint4 *>(stage + rr * RB + ((cc ^ (rr & (CH - 1))) * 16));
                 const int grow = q0 + t * BM + quad * 32 + rr;
@@ -985,22 +1368,33 @@ echo_status launch_items_dh(const void *Q, int64_t ldq, const void *K, const voi
 
 constexpr int kSplitMax = 8;   // CTAs of a cluster (portable size)
 
-// attn_tc_kernel may take its dynamic shared memory (once per device)
+// the one-shot kernel of a head size
+template <int DH, bool SPLIT>
+constexpr auto one_shot_kernel() {
+    if constexpr (DH == 64) return attn_d64_kernel<SPLIT>;
+    else return attn_tc_kernel<DH, SPLIT>;
+}
+template <int DH>
+constexpr int one_shot_threads() { return DH == 64 ? D64_THREADS : THREADS; }
+template <int DH>
+constexpr int one_shot_smem() { return DH == 64 ? D64_SMEM : Cfg<DH>::SMEM; }
+
+// it may take its dynamic shared memory (once per device)
 template <int DH>
 void raise_smem_cap() {
     static int attr_done[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-        cudaFuncSetAttribute(attn_tc_kernel<DH, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             Cfg<DH>::SMEM);
-        cudaFuncSetAttribute(attn_tc_kernel<DH, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             Cfg<DH>::SMEM);
+        cudaFuncSetAttribute(one_shot_kernel<DH, false>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             one_shot_smem<DH>());
+        cudaFuncSetAttribute(one_shot_kernel<DH, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             one_shot_smem<DH>());
         attr_done[dev] = 1;
     }
 }
 
-// CTAs of attn_tc_kernel<DH, true> that run at once in clusters of `splits`, on the
+// CTAs of the splitting one-shot kernel that run at once in clusters of `splits`, on the
 // current device (one CTA per SM; clusters of 4 and 8 leave a few SMs idle)
 template <int DH>
 int split_slots(int splits) {
@@ -1013,8 +1407,8 @@ int split_slots(int splits) {
         raise_smem_cap<DH>();
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(splits * num_sms()), 1, 1);
-        cfg.blockDim = dim3(THREADS, 1, 1);
-        cfg.dynamicSmemBytes = Cfg<DH>::SMEM;
+        cfg.blockDim = dim3(one_shot_threads<DH>(), 1, 1);
+        cfg.dynamicSmemBytes = one_shot_smem<DH>();
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = (unsigned)splits;
@@ -1022,7 +1416,7 @@ int split_slots(int splits) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int c = 0;
-        if (cudaOccupancyMaxActiveClusters(&c, attn_tc_kernel<DH, true>, &cfg) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveClusters(&c, one_shot_kernel<DH, true>(), &cfg) != cudaSuccess) {
             (void)cudaGetLastError();
             c = 0;
         }
@@ -1035,11 +1429,11 @@ int split_slots(int splits) {
 // active latents still fill the SMs: the fewest key-block times (1.2 us),
 // counted as waves of CTAs times the blocks of one CTA plus its fixed cost
 // (set-up and epilogue 4; with the sum over the cluster 7).  Measured, one CTA
-// against the split chosen: 389 queries x 7801 keys, 16 heads of 64: 80.7 ->
-// 29.6 us (4); 130 x 2000 x 6 heads of 64: 23.1 -> 10.8 us (8); 600 x 2000 x 16
-// heads of 64: 23.7 -> 16.9 us (2); 3198 x 63960 x 40 heads of 128 (3.4 waves):
-// 2.71 -> 2.60 ms under the power cap (2).  At 1560 x 7800 x 16 (0.74 waves) two take
-// 89 us against 76 and the rule stays at one.
+// against the split chosen: 389 queries x 7801 keys, 16 heads of 64: 61 -> 23 us
+// (4); 130 x 2000 x 6 heads of 64: 21.4 -> 10.2 us (8); 600 x 2000 x 16 heads of
+// 64: 22.0 -> 14.1 us (2); 3198 x 63960 x 40 heads of 128 (3.4 waves): 2.71 ->
+// 2.60 ms under the power cap (2).  At 1560 x 7800 x 16 (0.74 waves) two take
+// 72 us against 62 and the rule stays at one.
 template <int DH>
 int choose_splits(int64_t items, int nb) {
     int best = 1;
@@ -1074,15 +1468,15 @@ echo_status launch_dh(const void *Q, int64_t ldq, const void *K, const void *V, 
     const int ntp = (M + TILES * BM - 1) / (TILES * BM);
     if (splits == 1) {
         echo::LaunchScope ls(ECHO_K_ATTENTION, M, L, (int64_t)H * DH, st);
-        echo::launch_chained(attn_tc_kernel<DH, false>, dim3(ntp, H), dim3(THREADS),
-                             Cfg<DH>::SMEM, st,
-                             tq, tk, tv, p);
+        echo::launch_chained(one_shot_kernel<DH, false>(), dim3(ntp, H), dim3(one_shot_threads<DH>()),
+                             one_shot_smem<DH>(), st, tq, tk, tv, p);
         return echo::last_launch_status();
     }
     echo::LaunchScope ls(ECHO_K_ATTENTION, M, L, (int64_t)H * DH, st);
-    if (echo::launch_chained_cluster((unsigned)splits, attn_tc_kernel<DH, true>,
-                                     dim3((unsigned)(ntp * splits), (unsigned)H), dim3(THREADS),
-                                     Cfg<DH>::SMEM, st, tq, tk, tv, p) != cudaSuccess)
+    if (echo::launch_chained_cluster((unsigned)splits, one_shot_kernel<DH, true>(),
+                                     dim3((unsigned)(ntp * splits), (unsigned)H),
+                                     dim3(one_shot_threads<DH>()), one_shot_smem<DH>(), st, tq, tk,
+                                     tv, p) != cudaSuccess)
         return ECHO_ERR_CUDA;
     return echo::last_launch_status();
 }

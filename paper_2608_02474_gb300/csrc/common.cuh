@@ -463,6 +463,25 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
            | ((uint32_t)(M >> 4) << 24);     // M / 16
 }
 
+// Barrier `id` (1..15) among `threads` threads of the CTA, whole warps.
+ECHO_DEV void named_bar_sync(int id, int threads) {
+    asm volatile("barrier.cta.sync.aligned %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// The same barrier; returns whether `v` holds in any of its threads.
+ECHO_DEV bool named_bar_or(int id, int threads, bool v) {
+    uint32_t any;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %3, 0;\n\t"
+        "barrier.cta.red.or.pred.aligned q, %1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(any)
+        : "r"(id), "r"(threads), "r"((uint32_t)v)
+        : "memory");
+    return any != 0;
+}
+
 ECHO_DEV bool elect_one_sync() {
     uint32_t pred = 0;
     asm volatile(

@@ -49,11 +49,30 @@ def check(ec, Q, KV, H, d):
     (256, 2500, 19, 128),    # 4 or 8 CTAs, whole tiles
     (600, 1999, 16, 128),    # 2 CTAs
     (1100, 900, 12, 64),     # 2 CTAs, 8 blocks
+    (300, 2049, 40, 64),     # one CTA per tile pair, the last block of one key
+    (257, 2200, 76, 64),     # 152 CTAs, an odd number of blocks
 ])
 def test_attention_split_keys(ec, M, L, H, d):
     D = H * d
     check(ec, G.random_rows(M, D, seed=M + d, scale=1.5),
           G.random_rows(L, 2 * D, seed=L + d, scale=1.5), H, d)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("H", [2, 40])       # keys split over a cluster; one CTA per tile pair
+def test_attention_late_maxima(ec, d, H):
+    """Keys whose logits exceed the first block's by far more than 2^64 in one half
+    of a later block only: the rescale path, which both halves of a row take."""
+    M, L = 300, 2100
+    D = H * d
+    g = np.random.default_rng(d + H)
+    Q = np.full((M, D), 2.0, dtype=F32) + g.standard_normal((M, D)).astype(F32) * F32(0.05)
+    K = g.standard_normal((L, D)).astype(F32) * F32(0.1)
+    K[700:710] += F32(3.0)
+    K[1500:1505] += F32(6.0)
+    V = g.standard_normal((L, D)).astype(F32)
+    Q, K, V = (G.to_bf16_values(a) for a in (Q, K, V))
+    check(ec, Q, np.concatenate([K, V], axis=1), H, d)
 
 
 @pytest.mark.parametrize("d", [64, 128])
