@@ -315,8 +315,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             tc_fence_after();
             if (leader) {
                 mma_pv(1, vs, acc0);
-                if (!more) tc_commit(&pv_done[1]);
                 tc_commit(&ring_empty[vs]);                      // V_j no longer needed
+                if (!more) tc_commit(&pv_done[1]);               // the last arrival of all
                 if (more) {
                     mma_s(1, ns);
                     tc_commit(&s_full[1]);
@@ -537,7 +537,7 @@ attn_d64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     // Every barrier is reused only after its previous phase has been observed
     // by its waiter, so no waiter can fall two phases behind.
     __shared__ __align__(8) uint64_t q_full, ring_full[RING_MAX], ring_empty[RING_MAX];
-    __shared__ __align__(8) uint64_t s_full[S_BUFS], p_full[S_BUFS], pv_done[TILES];
+    __shared__ __align__(8) uint64_t s_full[S_BUFS], p_full[S_BUFS], pv_done[TILES], o_done[TILES];
     __shared__ __align__(8) uint64_t drain;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
@@ -558,7 +558,10 @@ attn_d64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             mbar_init(&s_full[b], 1);
             mbar_init(&p_full[b], 8);    // one arrival per softmax warp of the tile
         }
-        for (int t = 0; t < TILES; ++t) mbar_init(&pv_done[t], 1);
+        for (int t = 0; t < TILES; ++t) {
+            mbar_init(&pv_done[t], 1);   // P V of every block: for a rescale of O
+            mbar_init(&o_done[t], 1);    // P V of the last block
+        }
         mbar_init(&drain, 1);
         abort_flag = 0;
         fence_barrier_init();
@@ -668,8 +671,9 @@ attn_d64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             tc_fence_after();
             if (leader) {
                 mma_pv(k & 1, buf, vs, k > 1 ? 1u : 0u);
-                tc_commit(&pv_done[k & 1]);
                 if (k & 1) tc_commit(&ring_empty[vs]);           // K_j and V_j no longer needed
+                tc_commit(&pv_done[k & 1]);
+                if (k + 2 >= items) tc_commit(&o_done[k & 1]);   // the last arrival of all
             }
             __syncwarp();
             if ((k & 1) && ++vs == RING) vs = 0;
@@ -792,7 +796,8 @@ attn_d64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                     l *= alpha;
                     m_used = m_new;
                 }
-                if (j > 0) {   // O_t is settled once P V of the block before is done
+                if (j > 0) {   // O_t is settled once P V of the block before is done (the
+                               // one before that is: S of this item was issued after it)
                     mbar_wait(&pv_done[t], (j - 1) & 1, abort_v, p.err);
                     __syncwarp();
                     tc_fence_after();
@@ -823,7 +828,9 @@ attn_d64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             if (lane == 0) mbar_arrive(&p_full[buf]);
             if ((buf += 2) >= S_BUFS) { buf -= S_BUFS; sph ^= 1u; }
         }
-        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&pv_done[t], (nb - 1) & 1, abort_v, p.err));
+        // a barrier of its own: on pv_done, with a phase a block, the last phase's parity
+        // could be taken for that of the last but two while two P V are under way
+        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&o_done[t], 0, abort_v, p.err));
         if (ok) tc_fence_after();
         ok = !named_bar_or(bar_id, 64, !ok);                 // both warps of the rows, or neither
         row_x[t][half][row] = l;                             // the row's sum over both halves
@@ -1105,8 +1112,8 @@ attn_items_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             tc_fence_after();
             if (leader) {
                 mma_pv(1, vs, acc0);
-                if (last_j) tc_commit(&pv_done[1]);
                 tc_commit(&ring_empty[vs]);
+                if (last_j) tc_commit(&pv_done[1]);
                 if (more) {
                     mma_s(kn & 1, 1, ns);
                     tc_commit(&s_full[1]);
