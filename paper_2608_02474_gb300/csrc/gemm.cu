@@ -256,6 +256,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     const int num_kb = p.Kd / BK;
     const int num_m = (p.M + 2 * BM - 1) / (2 * BM), num_n = (p.N + BN - 1) / BN;
     const int num_tiles = num_m * num_n;
+    // Arrivals that nothing waits for are left out (the ring slots of the last
+    // STAGES k-blocks, the accumulators of the last two tiles): they may land after
+    // this CTA has left, on the barriers that the next kernel has set up there.
+    const int my_tiles = (num_tiles - pair + num_pairs - 1) / num_pairs;
+    const int my_kbs = my_tiles * num_kb;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -354,7 +359,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     for (int k = 0; k < BK / 16; ++k)
                         tc_mma_pair_f16(d_tmem, desc(a_lo + 2 * k), desc(b_lo + 2 * k), C::IDESC,
                                         (kb | k) != 0);
-                    tc_commit_pair(&empty_bar[s], 0x3);   // the stage is free in both CTAs
+                    if (it + STAGES < my_kbs)
+                        tc_commit_pair(&empty_bar[s], 0x3);   // the stage is free in both CTAs
                 }
                 __syncwarp();
             }
@@ -391,7 +397,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 [&]() {
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive_remote_relaxed(empty_even[buf]);
+                    if (lane == 0 && local + 2 < my_tiles) mbar_arrive_remote_relaxed(empty_even[buf]);
                 });
             if (!ok) break;
         }
