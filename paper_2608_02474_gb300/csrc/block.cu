@@ -6,7 +6,7 @@
 //   LN          n1 = LN(x), all NT rows; the active rows are also written to
 //               na = LN(x[idx]) through the row map  ("select active latents")
 //   GEMM        KV = n1 [Wk; Wv]^T + [bk; bv]          (K, V over all latents)
-//   GEMM        Q' = na Wq^T + bq
+//               Q' = na Wq^T + bq                      (one launch)
 //   attention   att = MHA(Q', K, V)
 //   GEMM        h1 = att Wo^T + bo + x[idx]             (fp32)
 //   LN, GEMM    Qc = LN(h1) Wqc^T + bqc
@@ -99,16 +99,14 @@ echo_status check_block(const echo_block_weights *w, const echo_block_dims *dims
     return ECHO_OK;
 }
 
-// K/V of the rows listed in rows_a and rows_b (either may be empty; a row in
-// both is computed twice, to the same bits): the list [rows_a; rows_b] at
-// ws + L.rows, the rows' layer norm into ws + L.n1 (compact, in that order),
-// their K/V scattered into kv.
-echo_status refresh_kv_rows(const echo_block_weights *w, const echo_block_dims &d,
-                            const void *x, const int32_t *rows_a, int32_t n_a,
-                            const int32_t *rows_b, int32_t n_b, void *kv, uint8_t *ws,
-                            const Layout &L, cudaStream_t st) {
+// The rows listed in rows_a and rows_b (either may be empty; a row in both is
+// computed twice, to the same bits), ready for their K/V projection: the list
+// [rows_a; rows_b] at ws + L.rows, the rows' layer norm into ws + L.n1 (compact,
+// in that order).
+echo_status norm_kv_rows(const echo_block_dims &d, const void *x, const int32_t *rows_a, int32_t n_a,
+                         const int32_t *rows_b, int32_t n_b, uint8_t *ws, const Layout &L,
+                         cudaStream_t st) {
     using namespace echo;
-    const int D = d.D;
     int32_t *rows = reinterpret_cast<int32_t *>(ws + L.rows);
     const int n = n_a + n_b;
     if (n == 0) return ECHO_OK;
@@ -118,10 +116,17 @@ echo_status refresh_kv_rows(const echo_block_weights *w, const echo_block_dims &
     if (n_b > 0 && cudaMemcpyAsync(rows + n_a, rows_b, sizeof(int32_t) * (size_t)n_b,
                                    cudaMemcpyDeviceToDevice, st) != cudaSuccess)
         return ECHO_ERR_CUDA;
-    launch_layernorm(x, ECHO_BF16, rows, n, D, ws + L.n1, st);
-    LinearArgs a{ws + L.n1, D, n, D, w->Wkv, w->bkv, 2 * D, 0, nullptr, ECHO_BF16, nullptr, kv,
-                 2 * (int64_t)D, ECHO_BF16};
-    a.out_rows = rows;
+    launch_layernorm(x, ECHO_BF16, rows, n, d.D, ws + L.n1, st);
+    return last_launch_status();
+}
+
+// their K/V, scattered into kv
+echo_status project_kv_rows(const echo_block_weights *w, const echo_block_dims &d, int32_t n, void *kv,
+                            uint8_t *ws, const Layout &L, cudaStream_t st) {
+    using namespace echo;
+    LinearArgs a{ws + L.n1, d.D, n, d.D, w->Wkv, w->bkv, 2 * d.D, 0, nullptr, ECHO_BF16, nullptr, kv,
+                 2 * (int64_t)d.D, ECHO_BF16};
+    a.out_rows = reinterpret_cast<const int32_t *>(ws + L.rows);
     return launch_linear(a, st);
 }
 
@@ -137,13 +142,13 @@ echo_status refresh_kv_all(const echo_block_weights *w, const echo_block_dims &d
 
 // rowmap and the block on the K active rows: y_act (bf16 [K, D]) at ws + L.yact,
 // or, with y_scatter, straight into rows idx[j] of y_scatter.  With kv_ext the
-// K/V of every row come from (and, unless kv_ready, go to) the caller's buffer;
-// kv_ready: it is already up to date, and only the active rows are normalised
-// (gathered into na) for Q'.
+// K/V of every row live in the caller's buffer.  n_kv_rows < 0: they are computed
+// here; else only those of the n_kv_rows rows that norm_kv_rows has prepared (K 0:
+// by the caller), and only the active rows are normalised (gathered into na).
 echo_status run_active(const echo_block_weights *w, const echo_block_dims &d, const void *x,
                        const int32_t *idx, int32_t K, uint8_t *ws, const Layout &L,
                        cudaStream_t st, void *y_scatter = nullptr, void *kv_ext = nullptr,
-                       bool kv_ready = false) {
+                       int32_t n_kv_rows = -1) {
     using namespace echo;
     const int NT = d.T * d.N;
     int32_t *rowmap = reinterpret_cast<int32_t *>(ws + L.rowmap);
@@ -158,17 +163,22 @@ echo_status run_active(const echo_block_weights *w, const echo_block_dims &d, co
     uint32_t *amax = reinterpret_cast<uint32_t *>(ws + L.amax);
     launch_rowmap(idx, K, NT, rowmap, amax, K, st);
     if (K > 0) {
-        if (kv_ready) {
+        // Q' and the K/V that are not there yet in one launch: alone, the few tiles of
+        // Q' would leave most SM pairs idle (7800 tokens, D 1024, K 1560: 36 -> 29 us)
+        const LinearArgs qproj{na, D, K, D, w->Wq, w->bq, D, 0, nullptr, ECHO_BF16, nullptr, qa, D,
+                               ECHO_BF16};
+        if (n_kv_rows >= 0) {
             launch_layernorm(x, ECHO_BF16, idx, K, D, na, st);   // the active rows only
+            LinearArgs kvproj{n1, D, n_kv_rows, D, w->Wkv, w->bkv, 2 * D, 0, nullptr, ECHO_BF16,
+                              nullptr, kv, 2 * (int64_t)D, ECHO_BF16};
+            kvproj.out_rows = reinterpret_cast<const int32_t *>(ws + L.rows);
+            s = launch_linear_pair(kvproj, qproj, st);
         } else {
             // LN over every latent; the active rows also land in na, gathered
             launch_layernorm_scatter(x, NT, D, n1, rowmap, na, st);
-            s = launch_linear({n1, D, NT, D, w->Wkv, w->bkv, 2 * D, 0, nullptr, ECHO_BF16, nullptr,
-                               kv, 2 * (int64_t)D, ECHO_BF16}, st);
-            if (s != ECHO_OK) return s;
+            s = launch_linear_pair({n1, D, NT, D, w->Wkv, w->bkv, 2 * D, 0, nullptr, ECHO_BF16,
+                                    nullptr, kv, 2 * (int64_t)D, ECHO_BF16}, qproj, st);
         }
-        s = launch_linear({na, D, K, D, w->Wq, w->bq, D, 0, nullptr, ECHO_BF16, nullptr, qa, D,
-                           ECHO_BF16}, st);
         if (s != ECHO_OK) return s;
         s = launch_attention(qa, D, kvb, kvb + D, 2 * (int64_t)D, K, NT, d.H, d.d, att, D, st);
         if (s != ECHO_OK) return s;
@@ -261,13 +271,12 @@ extern "C" echo_status echo_block_step_kv(const echo_block_weights *w, const ech
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     uint8_t *ws = static_cast<uint8_t *>(workspace);
     if (kv_valid) {
-        s = refresh_kv_rows(w, d, x, rows_a, n_a, rows_b, n_b, kv, ws, L, st);
-        if (s == ECHO_OK) s = run_active(w, d, x, idx, K, ws, L, st, y, kv, true);
-    } else if (K > 0) {
-        s = run_active(w, d, x, idx, K, ws, L, st, y, kv, false);
+        s = norm_kv_rows(d, x, rows_a, n_a, rows_b, n_b, ws, L, st);
+        if (s == ECHO_OK && K == 0) s = project_kv_rows(w, d, n_a + n_b, kv, ws, L, st);
+        if (s == ECHO_OK) s = run_active(w, d, x, idx, K, ws, L, st, y, kv, n_a + n_b);
     } else {
-        s = refresh_kv_all(w, d, x, kv, ws, L, st);
-        if (s == ECHO_OK) s = run_active(w, d, x, idx, K, ws, L, st, y, kv, true);
+        if (K == 0) s = refresh_kv_all(w, d, x, kv, ws, L, st);
+        if (s == ECHO_OK) s = run_active(w, d, x, idx, K, ws, L, st, y, kv);
     }
     if (s != ECHO_OK) return s;
     const int32_t *rowmap = reinterpret_cast<const int32_t *>(ws + L.rowmap);

@@ -236,10 +236,13 @@ ECHO_DEV bool epilogue_rows(const GemmParams &p, uint32_t tacc, uint8_t *stage, 
     return true;
 }
 
-template <int EPI, int BN>
+// DUAL: a second projection of the same depth (A2 W2^T, p2) continues the tile
+// list; its tiles fill the wave that the first one's leave part empty.
+template <int EPI, int BN, bool DUAL>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-            const GemmParams p) {
+            const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
+            const __grid_constant__ GemmParams p, const __grid_constant__ GemmParams p2) {
     using C = Cfg<BN>;
     constexpr int STAGES = C::STAGES, STAGE_BYTES = C::STAGE_BYTES;
     extern __shared__ uint8_t smem_raw[];
@@ -255,7 +258,14 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
     const int num_kb = p.Kd / BK;
     const int num_m = (p.M + 2 * BM - 1) / (2 * BM), num_n = (p.N + BN - 1) / BN;
-    const int num_tiles = num_m * num_n;
+    const int tiles1 = num_m * num_n;
+    const int num_m2 = DUAL ? (p2.M + 2 * BM - 1) / (2 * BM) : 0;
+    const int num_n2 = DUAL ? (p2.N + BN - 1) / BN : 0;
+    const int num_tiles = tiles1 + num_m2 * num_n2;
+    auto coords = [&](int t, int &mt, int &nt) {
+        if (DUAL && t >= tiles1) tile_coords<BN>(t - tiles1, num_m2, num_n2, mt, nt);
+        else tile_coords<BN>(t, num_m, num_n, mt, nt);
+    };
     // Arrivals that nothing waits for are left out (the ring slots of the last
     // STAGES k-blocks, the accumulators of the last two tiles): they may land after
     // this CTA has left, on the barriers that the next kernel has set up there.
@@ -276,6 +286,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         fence_barrier_init();
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
+        if (DUAL) {
+            tma_prefetch_desc(&tmA2);
+            tma_prefetch_desc(&tmB2);
+        }
     }
     cluster_sync_all();   // both CTAs' barriers exist before any arrival from the other CTA
     if (warp == 2) tmem_alloc_pair(&tmem_slot, C::TMEM_COLS);
@@ -296,7 +310,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         bool ok = true;
         for (int t = pair; ok && t < num_tiles; t += num_pairs) {
             int mt, nt;
-            tile_coords<BN>(t, num_m, num_n, mt, nt);
+            coords(t, mt, nt);
+            const CUtensorMap *ma = DUAL && t >= tiles1 ? &tmA2 : &tmA;
+            const CUtensorMap *mb = DUAL && t >= tiles1 ? &tmB2 : &tmB;
             for (int kb = 0; kb < num_kb; ++kb, ++it) {
                 const int s = it % STAGES;
                 if (!mbar_wait_cluster(&empty_bar[s], ((it / STAGES) & 1) ^ 1, abort_v, p.err)) {
@@ -306,8 +322,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 uint8_t *a = smem + s * STAGE_BYTES;
                 const uint32_t bar = full0 + (uint32_t)(s * sizeof(uint64_t));
                 if (rank == 0) mbar_arrive_expect_tx(&full_bar[s], 2 * STAGE_BYTES);
-                tma_load_2d_pair(a, &tmA, bar, kb * BK, mt * 2 * BM + (int)rank * BM);
-                tma_load_2d_pair(a + A_BYTES, &tmB, bar, kb * BK, nt * BN + (int)rank * (BN / 2));
+                tma_load_2d_pair(a, ma, bar, kb * BK, mt * 2 * BM + (int)rank * BM);
+                tma_load_2d_pair(a + A_BYTES, mb, bar, kb * BK, nt * BN + (int)rank * (BN / 2));
             }
         }
         if (*abort_v) {  // let this CTA's copies land before it exits
@@ -383,9 +399,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         for (int t = pair; t < num_tiles; t += num_pairs, ++local) {
             const int buf = local & 1;
             int mt, nt;
-            tile_coords<BN>(t, num_m, num_n, mt, nt);
+            coords(t, mt, nt);
             const bool ok = epilogue_rows<EPI, BN / 2>(
-                p, tmem + lane_base + (uint32_t)(buf * BN + half * (BN / 2)), stage,
+                DUAL && t >= tiles1 ? p2 : p, tmem + lane_base + (uint32_t)(buf * BN + half * (BN / 2)), stage,
                 mt * 2 * BM + (int)rank * BM + q * 32, nt * BN + half * (BN / 2),
                 [&]() {
                     const bool w = __all_sync(0xffffffffu,
@@ -423,14 +439,20 @@ int num_sms() {
     return cached[dev];
 }
 
-template <int EPI, int BN>
-echo_status run_bn(const CUtensorMap &ta, const CUtensorMap &tb, const GemmParams &p, cudaStream_t st) {
+// tensor maps and parameters of one projection
+struct Problem {
+    CUtensorMap a, b;
+    GemmParams p;
+};
+
+template <int EPI, int BN, bool DUAL>
+echo_status run_bn(const Problem &x, const Problem &y, cudaStream_t st) {
     static int pairs_max[64] = {};   // per device: co-resident CTA pairs (0: not set up yet)
     constexpr int SMEM_BYTES = Cfg<BN>::SMEM_BYTES;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return ECHO_ERR_CUDA;
     if (!pairs_max[dev]) {   // a benign race computes the same value twice
-        if (cudaFuncSetAttribute(gemm_kernel<EPI, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(gemm_kernel<EPI, BN, DUAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  SMEM_BYTES) != cudaSuccess)
             return ECHO_ERR_CUDA;
         cudaLaunchConfig_t cfg = {};
@@ -438,15 +460,20 @@ echo_status run_bn(const CUtensorMap &ta, const CUtensorMap &tb, const GemmParam
         cfg.blockDim = dim3(THREADS, 1, 1);
         cfg.dynamicSmemBytes = SMEM_BYTES;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, gemm_kernel<EPI, BN>, &cfg) != cudaSuccess || n < 1)
+        if (cudaOccupancyMaxActiveClusters(&n, gemm_kernel<EPI, BN, DUAL>, &cfg) != cudaSuccess || n < 1)
             return ECHO_ERR_CUDA;
         pairs_max[dev] = n;
     }
-    const int tiles = ((p.M + 2 * BM - 1) / (2 * BM)) * ((p.N + BN - 1) / BN);
+    auto tiles_of = [](const GemmParams &p) {
+        return ((p.M + 2 * BM - 1) / (2 * BM)) * ((p.N + BN - 1) / BN);
+    };
+    const int tiles = tiles_of(x.p) + (DUAL ? tiles_of(y.p) : 0);
     const int pairs = tiles < pairs_max[dev] ? tiles : pairs_max[dev];
-    echo::LaunchScope ls(ECHO_K_GEMM, p.M, p.N, p.Kd, st);
-    echo::launch_chained(gemm_kernel<EPI, BN>, dim3(2 * pairs), dim3(THREADS), SMEM_BYTES, st,
-                         ta, tb, p);
+    // two projections count as one with the rows that give the same operations
+    const int64_t m = x.p.M + (DUAL ? (int64_t)y.p.M * y.p.N / x.p.N : 0);
+    echo::LaunchScope ls(ECHO_K_GEMM, m, x.p.N, x.p.Kd, st);
+    echo::launch_chained(gemm_kernel<EPI, BN, DUAL>, dim3(2 * pairs), dim3(THREADS), SMEM_BYTES, st, x.a,
+                         x.b, y.a, y.b, x.p, y.p);
     return echo::last_launch_status();
 }
 
@@ -457,30 +484,16 @@ echo_status run_bn(const CUtensorMap &ta, const CUtensorMap &tb, const GemmParam
 // 10.3 us, 1560 x 1024 x 4096 25.7 -> 21.4 us, 400 x 640 x 2048 16.8 -> 13.4 us,
 // 1563 x 4096 x 1024 25.5 -> 23.2 us; at 7800 x 1024 x 4096 they take 69 us
 // against 48, at 600 x 5120 x 5120 44 against 31, and the rule keeps 256.
-bool narrow_tiles(int M, int N, int Kd) {
-    const int64_t pairs = num_sms() / 2, nm = (M + 2 * BM - 1) / (2 * BM), kb = Kd / BK;
-    const int64_t w256 = (nm * ((N + 255) / 256) + pairs - 1) / pairs;
-    const int64_t w128 = (nm * ((N + 127) / 128) + pairs - 1) / pairs;
+bool narrow_tiles(int M, int N, int Kd, int M2 = 0, int N2 = 0) {
+    const int64_t pairs = num_sms() / 2, kb = Kd / BK;
+    const int64_t nm = (M + 2 * BM - 1) / (2 * BM), nm2 = (M2 + 2 * BM - 1) / (2 * BM);
+    const int64_t w256 = (nm * ((N + 255) / 256) + nm2 * ((N2 + 255) / 256) + pairs - 1) / pairs;
+    const int64_t w128 = (nm * ((N + 127) / 128) + nm2 * ((N2 + 127) / 128) + pairs - 1) / pairs;
     return w128 * (kb * 340 + 600) + 1500 < w256 * (kb * 512 + 600) + 3000;
 }
 
-template <int EPI>
-echo_status run(const echo::LinearArgs &a, const GemmParams &p, cudaStream_t st) {
-    const bool narrow = narrow_tiles(p.M, p.N, p.Kd);
-    CUtensorMap ta, tb;
-    if (!echo::make_tmap_bf16(&ta, a.A, (uint64_t)a.M, (uint64_t)a.Kd, (uint64_t)a.lda, BM) ||
-        !echo::make_tmap_bf16(&tb, a.W, (uint64_t)a.N, (uint64_t)a.Kd, (uint64_t)a.Kd, narrow ? 64 : 128))
-        return ECHO_ERR_CUDA;
-    return narrow ? run_bn<EPI, 128>(ta, tb, p, st) : run_bn<EPI, 256>(ta, tb, p, st);
-}
-
-}  // namespace
-
-namespace echo {
-
-echo_status launch_linear(const LinearArgs &a, cudaStream_t st) {
-    if (a.M <= 0) return ECHO_OK;
-    GemmParams p;
+bool make_problem(const echo::LinearArgs &a, bool narrow, Problem &x) {
+    GemmParams &p = x.p;
     p.M = a.M; p.N = a.N; p.Kd = a.Kd;
     p.bias = static_cast<const __nv_bfloat16 *>(a.bias);
     p.resid = a.resid;
@@ -489,32 +502,63 @@ echo_status launch_linear(const LinearArgs &a, cudaStream_t st) {
     p.ldo = a.ldo;
     p.out_rows = a.out_rows;
     p.row_amax = a.row_amax;
-    p.err = device_error_ptr();
+    p.err = echo::device_error_ptr();
+    return echo::make_tmap_bf16(&x.a, a.A, (uint64_t)a.M, (uint64_t)a.Kd, (uint64_t)a.lda, BM) &&
+           echo::make_tmap_bf16(&x.b, a.W, (uint64_t)a.N, (uint64_t)a.Kd, (uint64_t)a.Kd,
+                                narrow ? 64 : 128);
+}
+
+template <int EPI>
+echo_status run(const echo::LinearArgs &a, cudaStream_t st) {
+    const bool narrow = narrow_tiles(a.M, a.N, a.Kd);
+    Problem x;
+    if (!make_problem(a, narrow, x)) return ECHO_ERR_CUDA;
+    return narrow ? run_bn<EPI, 128, false>(x, x, st) : run_bn<EPI, 256, false>(x, x, st);
+}
+
+}  // namespace
+
+namespace echo {
+
+echo_status launch_linear(const LinearArgs &a, cudaStream_t st) {
+    if (a.M <= 0) return ECHO_OK;
     int epi = 0;
     if (a.act == 1) epi |= EPI_GELU;
     if (a.resid) epi |= (a.resid_t == ECHO_BF16) ? EPI_RES_BF16 : EPI_RES_F32;
     if (a.out_t == ECHO_F32) epi |= EPI_OUT_F32;
     if (a.row_amax) {
         if (epi != EPI_RES_F32) return ECHO_ERR_INVALID_ARG;   // bf16 out, fp32 residual only
-        return run<EPI_RES_F32 | EPI_ROWAMAX>(a, p, st);
+        return run<EPI_RES_F32 | EPI_ROWAMAX>(a, st);
     }
     switch (epi) {
-        case 0: return run<0>(a, p, st);
-        case EPI_GELU: return run<EPI_GELU>(a, p, st);
-        case EPI_RES_BF16: return run<EPI_RES_BF16>(a, p, st);
-        case EPI_RES_F32: return run<EPI_RES_F32>(a, p, st);
-        case EPI_GELU | EPI_RES_BF16: return run<EPI_GELU | EPI_RES_BF16>(a, p, st);
-        case EPI_GELU | EPI_RES_F32: return run<EPI_GELU | EPI_RES_F32>(a, p, st);
-        case EPI_OUT_F32: return run<EPI_OUT_F32>(a, p, st);
-        case EPI_GELU | EPI_OUT_F32: return run<EPI_GELU | EPI_OUT_F32>(a, p, st);
-        case EPI_RES_BF16 | EPI_OUT_F32: return run<EPI_RES_BF16 | EPI_OUT_F32>(a, p, st);
-        case EPI_RES_F32 | EPI_OUT_F32: return run<EPI_RES_F32 | EPI_OUT_F32>(a, p, st);
+        case 0: return run<0>(a, st);
+        case EPI_GELU: return run<EPI_GELU>(a, st);
+        case EPI_RES_BF16: return run<EPI_RES_BF16>(a, st);
+        case EPI_RES_F32: return run<EPI_RES_F32>(a, st);
+        case EPI_GELU | EPI_RES_BF16: return run<EPI_GELU | EPI_RES_BF16>(a, st);
+        case EPI_GELU | EPI_RES_F32: return run<EPI_GELU | EPI_RES_F32>(a, st);
+        case EPI_OUT_F32: return run<EPI_OUT_F32>(a, st);
+        case EPI_GELU | EPI_OUT_F32: return run<EPI_GELU | EPI_OUT_F32>(a, st);
+        case EPI_RES_BF16 | EPI_OUT_F32: return run<EPI_RES_BF16 | EPI_OUT_F32>(a, st);
+        case EPI_RES_F32 | EPI_OUT_F32: return run<EPI_RES_F32 | EPI_OUT_F32>(a, st);
         case EPI_GELU | EPI_RES_BF16 | EPI_OUT_F32:
-            return run<EPI_GELU | EPI_RES_BF16 | EPI_OUT_F32>(a, p, st);
+            return run<EPI_GELU | EPI_RES_BF16 | EPI_OUT_F32>(a, st);
         case EPI_GELU | EPI_RES_F32 | EPI_OUT_F32:
-            return run<EPI_GELU | EPI_RES_F32 | EPI_OUT_F32>(a, p, st);
+            return run<EPI_GELU | EPI_RES_F32 | EPI_OUT_F32>(a, st);
     }
     return ECHO_ERR_INVALID_ARG;
+}
+
+echo_status launch_linear_pair(const LinearArgs &a, const LinearArgs &b, cudaStream_t st) {
+    if (a.M <= 0) return launch_linear(b, st);
+    if (b.M <= 0) return launch_linear(a, st);
+    if (a.Kd != b.Kd || a.act || b.act || a.resid || b.resid || a.row_amax || b.row_amax ||
+        a.out_t != ECHO_BF16 || b.out_t != ECHO_BF16)
+        return ECHO_ERR_INVALID_ARG;
+    const bool narrow = narrow_tiles(a.M, a.N, a.Kd, b.M, b.N);
+    Problem x, y;
+    if (!make_problem(a, narrow, x) || !make_problem(b, narrow, y)) return ECHO_ERR_CUDA;
+    return narrow ? run_bn<0, 128, true>(x, y, st) : run_bn<0, 256, true>(x, y, st);
 }
 
 }  // namespace echo

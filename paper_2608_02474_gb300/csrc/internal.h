@@ -90,6 +90,9 @@ struct LinearArgs {
     const int32_t *out_rows = nullptr;   // output row m is stored at row out_rows[m]
 };
 echo_status launch_linear(const LinearArgs &a, cudaStream_t st);
+// two projections of the same depth Kd in one launch; no activation or residual,
+// bf16 outputs (each may scatter its rows), neither reading what the other writes
+echo_status launch_linear_pair(const LinearArgs &a, const LinearArgs &b, cudaStream_t st);
 
 // attention.cu
 echo_status launch_attention(const void *Q, int64_t ldq, const void *K, const void *V, int64_t ldkv,
