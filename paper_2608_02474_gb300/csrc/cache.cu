@@ -2,8 +2,9 @@
 // and the mask fusion of Sec. 3.3 (active rows take the fresh block output,
 // every other row is reconstructed from the cache).
 //
-// quant_kernel: one warp per source row; pass 1 finds amax, pass 2 (served from
-//   L1/L2) writes the codes.  s = amax/127, inv = 127/amax, q = rint(v*inv)
+// quant_regs_kernel: one warp per source row, held in registers (bf16 up to 5120
+//   values); quant_kernel: pass 1 finds amax, pass 2 (served from L1/L2) writes
+//   the codes.  s = amax/127, inv = 127/amax, q = rint(v*inv)
 //   clamped to [-127, 127], all fp32 round-to-nearest: bit-exact by construction.
 // dequant kernels: one thread per 16 elements, 128-bit loads and stores.
 #include "common.cuh"
@@ -89,6 +90,55 @@ quant_kernel(const ST *__restrict__ src, const int32_t *__restrict__ rows, int n
     }
 }
 
+// The same for bf16 rows of up to 256 CPL values: the row is held packed in
+// registers (16-byte chunk lane + 32 k in v[k]), every load in flight at once, and
+// read once.  32760 rows of 5120: 114 us with two passes over the row, 93 us; 20000
+// rows of 2048: 30 -> 21 us.
+template <int CPL>
+__global__ void __launch_bounds__(kQuantThreads)
+quant_regs_kernel(const __nv_bfloat16 *__restrict__ src, const int32_t *__restrict__ rows, int n_rows,
+                  int D, int8_t *__restrict__ q, float *__restrict__ scale, int *err) {
+    pdl_enter();
+    const int lane = threadIdx.x & 31;
+    const int warps = kQuantThreads / 32;
+    const int C = D >> 3;
+    for (int j = blockIdx.x * warps + (threadIdx.x >> 5); j < n_rows; j += gridDim.x * warps) {
+        const uint4 *s = reinterpret_cast<const uint4 *>(src + (int64_t)j * D);
+        const int r = rows ? rows[j] : j;
+        uint4 v[CPL];
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) v[k] = lane + 32 * k < C ? __ldcs(s + lane + 32 * k) : make_uint4(0, 0, 0, 0);
+        const uint32_t ab = warp_amax_bf16<CPL>(v);
+        uint2 *qr = reinterpret_cast<uint2 *>(q + (int64_t)r * D);
+        const bool bad = ab >= 0x7F800000u;           // NaN or infinity in the row
+        const float amax = __uint_as_float(ab);
+        float sc = 0.f, inv = 0.f;
+        if (!bad && amax > 0.f) {
+            sc = __fdiv_rn(amax, 127.f);
+            inv = __fdiv_rn(127.f, amax);
+        }
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) {
+            if (lane + 32 * k >= C) continue;
+            float f[8];
+            unpack8_bf16(v[k], f);
+            qr[lane + 32 * k] = bad ? make_uint2(0, 0) : quant8(f, inv);
+        }
+        if (lane == 0) {
+            scale[r] = !bad ? sc : ab > 0x7F800000u ? __int_as_float(0x7fc00000) : INFINITY;
+            if (bad) echo_flag_error(err, ECHO_ERR_NONFINITE);
+        }
+    }
+}
+
+template <int CPL>
+void launch_quant_regs(const __nv_bfloat16 *src, const int32_t *rows, int n_rows, int D, int8_t *q,
+                       float *scale, int *err, cudaStream_t st) {
+    const int grid = (n_rows + kQuantThreads / 32 - 1) / (kQuantThreads / 32);
+    echo::launch_chained(quant_regs_kernel<CPL>, dim3(grid), dim3(kQuantThreads), 0, st, src, rows,
+                         n_rows, D, q, scale, err);
+}
+
 ECHO_DEV void dequant16(const int4 &qv, float s, float *f) {
     const int8_t *b = reinterpret_cast<const int8_t *>(&qv);
 #pragma unroll
@@ -117,16 +167,12 @@ __global__ void __launch_bounds__(kVecThreads)
 dequant_kernel(const int8_t *__restrict__ q, const float *__restrict__ scale,
                const int32_t *__restrict__ rows, int n_rows, int D, DT *__restrict__ dst) {
     pdl_enter();
-    const int C = D >> 4;
-    const int64_t total = (int64_t)n_rows * C;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int j = (int)(t / C), c = (int)(t % C);
-        const int r = rows ? rows[j] : j;
-        const int4 qv = __ldcs(reinterpret_cast<const int4 *>(q + (int64_t)r * D + 16 * c));
+    for (PieceWalk w(D >> 4); w.row < n_rows; w.next()) {
+        const int r = rows ? rows[w.row] : w.row;
+        const int4 qv = __ldcs(reinterpret_cast<const int4 *>(q + (int64_t)r * D + 16 * w.piece));
         float f[16];
         dequant16(qv, scale[r], f);
-        store16<DT>(dst + (int64_t)j * D + 16 * c, f);
+        store16<DT>(dst + (int64_t)w.row * D + 16 * w.piece, f);
     }
 }
 
@@ -156,12 +202,12 @@ dequant_merge_kernel(const int8_t *__restrict__ q, const float *__restrict__ sca
                      const int32_t *__restrict__ rowmap, const __nv_bfloat16 *__restrict__ y_act,
                      int NT, int D, __nv_bfloat16 *__restrict__ y) {
     pdl_enter();
-    const int C = D >> 4;
-    const int64_t total = (int64_t)NT * C;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(t / C), c = (int)(t % C);
-        const int pos = rowmap[i];
+    PieceWalk w(D >> 4);
+    int pos_next = w.row < NT ? rowmap[w.row] : 0;   // a step ahead of the piece's own loads
+    while (w.row < NT) {
+        const int i = w.row, c = w.piece, pos = pos_next;
+        w.next();
+        if (w.row < NT) pos_next = rowmap[w.row];
         uint4 *o = reinterpret_cast<uint4 *>(y + (int64_t)i * D + 16 * c);
         if (pos >= 0) {
             if (y_act) {
@@ -192,12 +238,12 @@ merge_quant_kernel(int8_t *__restrict__ q, float *__restrict__ scale,
                    const int32_t *__restrict__ rowmap, const uint32_t *__restrict__ amax_bits,
                    int NT, int D, __nv_bfloat16 *__restrict__ y, int *err) {
     pdl_enter();
-    const int C = D >> 4;
-    const int64_t total = (int64_t)NT * C;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(t / C), c = (int)(t % C);
-        const int pos = rowmap[i];
+    PieceWalk w(D >> 4);
+    int pos_next = w.row < NT ? rowmap[w.row] : 0;   // a step ahead of the piece's own loads
+    while (w.row < NT) {
+        const int i = w.row, c = w.piece, pos = pos_next;
+        w.next();
+        if (w.row < NT) pos_next = rowmap[w.row];
         uint4 *o = reinterpret_cast<uint4 *>(y + (int64_t)i * D + 16 * c);
         int4 *qr = reinterpret_cast<int4 *>(q + (int64_t)i * D + 16 * c);
         if (pos < 0) {
@@ -258,7 +304,14 @@ void launch_quant(const void *src, echo_dtype st_t, const int32_t *rows, int32_t
     (void)warps;
     int *err = device_error_ptr();
     LaunchScope ls(ECHO_K_QUANT, n_rows, D, 0, st);
-    if (st_t == ECHO_BF16)
+    const __nv_bfloat16 *b = static_cast<const __nv_bfloat16 *>(src);
+    if (st_t == ECHO_BF16 && D <= 1024)
+        launch_quant_regs<4>(b, rows, n_rows, D, q, scale, err, st);
+    else if (st_t == ECHO_BF16 && D <= 2048)
+        launch_quant_regs<8>(b, rows, n_rows, D, q, scale, err, st);
+    else if (st_t == ECHO_BF16 && D <= 5120)
+        launch_quant_regs<20>(b, rows, n_rows, D, q, scale, err, st);
+    else if (st_t == ECHO_BF16)
         echo::launch_chained(quant_kernel<__nv_bfloat16>, dim3(grid), dim3(kQuantThreads), 0, st,
             static_cast<const __nv_bfloat16 *>(src), rows, n_rows, D, q, scale, err);
     else

@@ -61,10 +61,64 @@ ECHO_DEV uint4 pack8_bf16(const float *f) {
     return u;
 }
 
+// A thread's walk over the pieces (row, piece of the row) of [n_rows, C] pieces in
+// steps of the whole grid, kept as row and piece: one division at the start instead
+// of a 64-bit division per piece, which was as long as moving the piece.
+struct PieceWalk {
+    int row, piece;
+    ECHO_DEV PieceWalk(int C) : C_(C) {
+        const unsigned t = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+        row = (int)(t / (unsigned)C);
+        piece = (int)(t % (unsigned)C);
+        rows_ = (int)(step / (unsigned)C);
+        pieces_ = (int)(step % (unsigned)C);
+    }
+    ECHO_DEV void next() {
+        row += rows_;
+        piece += pieces_;
+        if (piece >= C_) {
+            piece -= C_;
+            ++row;
+        }
+    }
+
+  private:
+    int C_, rows_, pieces_;
+};
+
 ECHO_DEV uint64_t globaltimer_ns() {
     uint64_t t;
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
     return t;
+}
+
+// max |v| of a warp's row of packed bf16 chunks as fp32 bits, in every lane: the bits
+// of non-negative floats order as integers, infinity above every number, NaN above it
+template <int CPL>
+ECHO_DEV uint32_t warp_amax_bf16(const uint4 *v) {
+    uint32_t lo = 0, hi = 0;
+#pragma unroll
+    for (int k = 0; k < CPL; ++k) {
+        const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            lo = max(lo, w[e] & 0x7FFFu);
+            hi = max(hi, w[e] & 0x7FFF0000u);
+        }
+    }
+    return __reduce_max_sync(0xffffffffu, max(lo << 16, hi));
+}
+
+// int8 codes of 8 values: clamp(rint(v inv), -127, 127)
+ECHO_DEV uint2 quant8(const float *f, float inv) {
+    uint32_t w[2] = {0u, 0u};
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        float t = rintf(__fmul_rn(f[k], inv));
+        t = fminf(fmaxf(t, -127.f), 127.f);
+        w[k >> 2] |= (uint32_t)(uint8_t)(int8_t)(int)t << (8 * (k & 3));
+    }
+    return make_uint2(w[0], w[1]);
 }
 
 // ---------------------------------------------------------------------------

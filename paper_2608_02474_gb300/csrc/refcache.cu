@@ -14,9 +14,9 @@
 //                8 rows and the last new reference carries into the next round;
 //   ref_alloc    one CTA ranks the new references in token order and hands
 //                them the free slots in slot order (block scans);
-//   ref_store    one warp per written row: a reference copies its row into its
-//                slot, a residual quantises x - r by the int8 rule, a run
-//                without a slot quantises x itself.
+//   ref_store    one CTA per written row (a warp above D = 8192): a reference
+//                copies its row into its slot, a residual quantises x - r by the
+//                int8 rule, a run without a slot quantises x itself.
 // Reconstruction (read, merge) is one thread per 16 values: bf16(r + q s).
 #include "common.cuh"
 #include "internal.h"
@@ -360,6 +360,89 @@ ref_store_kernel(const __nv_bfloat16 *__restrict__ src, const int32_t *__restric
     }
 }
 
+// The same for rows of up to 1024 CPL values, one CTA of 128 threads per row: the
+// row and its reference are held packed in registers (16-byte chunk tid + 128 k),
+// every load in flight at once, each read once.  One warp per row reading them in
+// two passes was bound by latency: 6552 residual rows of 5120 49 -> 31 us.
+constexpr int kRowThreads = 128;
+
+template <int CPL>
+__global__ void __launch_bounds__(kRowThreads)
+ref_store_row_kernel(const __nv_bfloat16 *__restrict__ src, const int32_t *__restrict__ rows, int n,
+                     int D, const int32_t *__restrict__ src_pos, const int32_t *__restrict__ slot_of,
+                     int8_t *__restrict__ q, float *__restrict__ scale, int32_t *__restrict__ ref,
+                     int32_t *refcount, __nv_bfloat16 *__restrict__ pool, int *err) {
+    __shared__ uint32_t warp_max[kRowThreads / 32];
+    pdl_enter();
+    const int tid = threadIdx.x;
+    const int C = D >> 3;
+    const int j = blockIdx.x;
+    const uint4 *vp = reinterpret_cast<const uint4 *>(src + (int64_t)j * D);
+    uint4 v[CPL], g[CPL];
+#pragma unroll
+    for (int k = 0; k < CPL; ++k)
+        v[k] = tid + kRowThreads * k < C ? __ldg(vp + tid + kRowThreads * k) : make_uint4(0, 0, 0, 0);
+    const int i = rows[j], jr = src_pos[j];
+    const int sl = slot_of[jr];
+    const bool is_ref = sl >= 0 && jr == j;
+    uint4 *pr = reinterpret_cast<uint4 *>(pool + (int64_t)(is_ref ? sl : 0) * D);
+    uint2 *qr = reinterpret_cast<uint2 *>(q + (int64_t)i * D);
+    // residual against the reference row, or the row itself without one; a new
+    // reference only looks for values that are not finite
+    const bool residual = sl >= 0 && !is_ref;
+    if (residual) {
+        const uint4 *rp = reinterpret_cast<const uint4 *>(src + (int64_t)jr * D);
+#pragma unroll
+        for (int k = 0; k < CPL; ++k)
+            g[k] = tid + kRowThreads * k < C ? __ldg(rp + tid + kRowThreads * k) : make_uint4(0, 0, 0, 0);
+    }
+    auto diff = [&](int k, float *f) {
+        unpack8_bf16(v[k], f);
+        if (residual) {
+            float r[8];
+            unpack8_bf16(g[k], r);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) f[e] = __fsub_rn(f[e], r[e]);
+        }
+    };
+    uint32_t ab = 0;   // max |x - r| as fp32 bits (NaN above infinity above every number)
+#pragma unroll
+    for (int k = 0; k < CPL; ++k) {
+        float f[8];
+        diff(k, f);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) ab = max(ab, __float_as_uint(f[e]) & 0x7FFFFFFFu);
+    }
+    ab = __reduce_max_sync(0xffffffffu, ab);
+    if ((tid & 31) == 0) warp_max[tid >> 5] = ab;
+    __syncthreads();
+    ab = max(max(warp_max[0], warp_max[1]), max(warp_max[2], warp_max[3]));
+    const bool bad = ab >= 0x7F800000u;
+    const float amax = __uint_as_float(ab);
+    float sc = 0.f, inv = 0.f;
+    if (!bad && amax > 0.f) {
+        sc = __fdiv_rn(amax, 127.f);
+        inv = __fdiv_rn(127.f, amax);
+    }
+#pragma unroll
+    for (int k = 0; k < CPL; ++k) {
+        const int c = tid + kRowThreads * k;
+        if (c >= C) continue;
+        if (is_ref) pr[c] = v[k];
+        float f[8];
+        diff(k, f);
+        qr[c] = is_ref || bad ? make_uint2(0, 0) : quant8(f, inv);
+    }
+    if (tid == 0) {
+        ref[i] = sl >= 0 ? sl : -1;
+        if (sl >= 0) atomicAdd(&refcount[sl], 1);
+        scale[i] = is_ref ? 0.f
+                   : !bad ? sc
+                          : ab > 0x7F800000u ? __int_as_float(0x7fc00000) : INFINITY;
+        if (bad) echo_flag_error(err, ECHO_ERR_NONFINITE);
+    }
+}
+
 // ---------------------------------------------------------------- reconstruction
 // 16 values of token i: bf16(r + float(q) s), r = 0 without a reference
 ECHO_DEV void ref_reconstruct16(const echo_cache &c, int i, int col, uint4 *out) {
@@ -401,11 +484,8 @@ __global__ void __launch_bounds__(kVec)
 cache_read_kernel(echo_cache c, const int32_t *__restrict__ rows, int n,
                   __nv_bfloat16 *__restrict__ dst) {
     pdl_enter();
-    const int C = c.D >> 4;
-    const int64_t total = (int64_t)n * C;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int j = (int)(t / C), col = 16 * (int)(t % C);
+    for (PieceWalk w(c.D >> 4); w.row < n; w.next()) {
+        const int j = w.row, col = 16 * w.piece;
         const int i = rows ? rows[j] : j;
         uint4 o[2];
         reconstruct16<KIND>(c, i, col, o);
@@ -421,11 +501,8 @@ __global__ void __launch_bounds__(kVec)
 cache_merge_kernel(echo_cache c, const int32_t *__restrict__ rowmap,
                    const __nv_bfloat16 *__restrict__ y_act, __nv_bfloat16 *__restrict__ y) {
     pdl_enter();
-    const int C = c.D >> 4;
-    const int64_t total = (int64_t)c.NT * C;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(t / C), col = 16 * (int)(t % C);
+    for (PieceWalk w(c.D >> 4); w.row < c.NT; w.next()) {
+        const int i = w.row, col = 16 * w.piece;
         const int pos = rowmap[i];
         uint4 *o = reinterpret_cast<uint4 *>(y + (int64_t)i * c.D + col);
         uint4 v[2];
@@ -446,12 +523,9 @@ __global__ void __launch_bounds__(kVec)
 cache_copy_kernel(const __nv_bfloat16 *__restrict__ src, const int32_t *__restrict__ rows, int n,
                   int D, __nv_bfloat16 *__restrict__ full, int *err) {
     pdl_enter();
-    const int C = D >> 3;
-    const int64_t total = (int64_t)n * C;
     bool bad = false;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int j = (int)(t / C), c = (int)(t % C);
+    for (PieceWalk w(D >> 3); w.row < n; w.next()) {
+        const int j = w.row, c = w.piece;
         const uint4 u = __ldcs(reinterpret_cast<const uint4 *>(src + (int64_t)j * D + 8 * c));
         bad |= bf16_nonfinite(u.x) || bf16_nonfinite(u.y) || bf16_nonfinite(u.z) ||
                bf16_nonfinite(u.w);
@@ -587,10 +661,23 @@ echo_status launch_cache_write(const echo_cache &c, const void *src, const int32
     if (last_launch_status() != ECHO_OK) return ECHO_ERR_CUDA;
     {
         LaunchScope ls(ECHO_K_REF_STORE, n, c.D, 0, st);
-        echo::launch_chained(ref_store_kernel, dim3(grid_for((int64_t)n * 32, kStoreThreads)),
-                             dim3(kStoreThreads), 0, st,
-            s, rows, n, c.D, w.src_pos, w.slot_of, c.q, c.scale, c.ref, c.refcount,
-            static_cast<__nv_bfloat16 *>(c.pool), err);
+        __nv_bfloat16 *pool = static_cast<__nv_bfloat16 *>(c.pool);
+        auto store_rows = [&](auto kernel) {
+            launch_chained(kernel, dim3(n), dim3(kRowThreads), 0, st, s, rows, n, c.D, w.src_pos,
+                           w.slot_of, c.q, c.scale, c.ref, c.refcount, pool, err);
+        };
+        if (c.D <= 1024)
+            store_rows(ref_store_row_kernel<1>);
+        else if (c.D <= 2048)
+            store_rows(ref_store_row_kernel<2>);
+        else if (c.D <= 5120)
+            store_rows(ref_store_row_kernel<5>);
+        else if (c.D <= 8192)
+            store_rows(ref_store_row_kernel<8>);
+        else
+            launch_chained(ref_store_kernel, dim3(grid_for((int64_t)n * 32, kStoreThreads)),
+                           dim3(kStoreThreads), 0, st, s, rows, n, c.D, w.src_pos, w.slot_of, c.q, c.scale, c.ref, c.refcount,
+                           pool, err);
     }
     return last_launch_status();
 }
