@@ -7,11 +7,12 @@
 //                decrement of the slot's count) and the bounds of each scan
 //                segment's written rows are recorded;
 //   ref_scan     one CTA per scan segment walks its written rows in token
-//                order, 8 rows a round: the rows are staged in shared memory,
-//                the 16 warps compute every fp32 cosine the walk can need (each
-//                row against the entering reference and against each earlier
-//                row of the round, canonical order), then one thread walks the
-//                8 rows and the last new reference carries into the next round;
+//                order, 6 rows a round: the rows are staged in shared memory,
+//                the 12 warps compute the fp32 cosines the walk is likely to need
+//                (each row against the entering reference and against the row
+//                before it, canonical order), then one thread walks the rows,
+//                asking for others where it must, and the last new reference
+//                carries into the next round;
 //   ref_alloc    one CTA ranks the new references in token order and hands
 //                them the free slots in slot order (block scans);
 //   ref_store    one CTA per written row (a warp above D = 8192): a reference
@@ -23,7 +24,8 @@
 
 namespace {
 
-constexpr int kScanWarps = 16;
+constexpr int kWin = 6;             // rows of a scan window
+constexpr int kScanWarps = 2 * kWin;
 constexpr int kAllocThreads = 1024;
 constexpr int kStoreThreads = 256;
 constexpr int kVec = 256;
@@ -95,25 +97,25 @@ ECHO_DEV void warp_dot(const uint4 *a, const uint4 *b, int C, int lane, bool nor
 // src_pos[j] = position (in rows) of row j's reference; j itself for a reference.
 //
 // One CTA per scan segment.  The segment's written rows are taken kWin at a
-// time: the window's rows are staged in shared memory, then the CTA computes
-// every similarity the walk over the window can need (each row against the
-// reference it entered with and against every earlier row of the window), and
-// one thread walks the window in order.  A window is resolved in one round
-// whatever the data.  Dynamic shared memory: kWin window rows, then the
-// current reference row (bf16, D each).
-constexpr int kWin = 8;
-constexpr int kPairs = kWin * (kWin + 1) / 2;
-
+// time: the window's rows are staged in shared memory, then every row is compared
+// with the reference that the window was entered with and with the row before it,
+// one similarity per warp, and one thread walks the window in order.  Those two
+// suffice while the reference stays or changes at every row; a row that follows a
+// change by two or more also needs its similarity to the row of the change, which
+// is then computed for the rest of the window at once before the walk goes on.
+// Dynamic shared memory: kWin window rows, then the current reference row (bf16, D
+// each); six rows leave room for three CTAs per SM at D = 5120.  6552 rows of 5120:
+// 70 us with all 36 similarities of windows of eight rows and two CTAs per SM, 49 us.
 __global__ void __launch_bounds__(kScanWarps * 32)
 ref_scan_kernel(const __nv_bfloat16 *__restrict__ src, const int32_t *__restrict__ seg_lo,
                 const int32_t *__restrict__ seg_hi, float tau, int D,
                 int32_t *__restrict__ src_pos) {
     pdl_enter();
     extern __shared__ uint4 s_buf[];
-    __shared__ float s_dot[kWin][kWin + 1];  // [w][t + 1], t = -1: the entering reference
+    __shared__ float s_dref[kWin], s_dprev[kWin], s_dcur[kWin];   // <w, ref>, <w, w - 1>, <w, s_cur>
     __shared__ float s_nv[kWin];
     __shared__ float s_nr;
-    __shared__ int s_jr, s_newref;
+    __shared__ int s_jr, s_cur, s_w, s_more;   // walk: reference row of the window (-1: entering), row
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int C = D >> 3;
     uint4 *ref = s_buf + (size_t)kWin * C;
@@ -138,68 +140,89 @@ ref_scan_kernel(const __nv_bfloat16 *__restrict__ src, const int32_t *__restrict
     __syncthreads();
     for (int j = lo + 1; j < hi; j += kWin) {
         const int nvalid = hi - j < kWin ? hi - j : kWin;
-        // stage the window's rows, four 16-byte loads in flight per thread
+        // stage the window's rows (consecutive in src), eight 16-byte loads in flight
         const int total = nvalid * C;
-        for (int b = threadIdx.x; b < total; b += 4 * (int)blockDim.x) {
-            uint4 u[4];
+        const uint4 *win = reinterpret_cast<const uint4 *>(src + (int64_t)j * D);
+        for (int b = threadIdx.x; b < total; b += 8 * (int)blockDim.x) {
+            uint4 u[8];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
+            for (int k = 0; k < 8; ++k) {
                 const int e = b + k * blockDim.x;
-                if (e < total) {
-                    const int w = e / C, c = e - w * C;
-                    u[k] = __ldg(reinterpret_cast<const uint4 *>(src + (int64_t)(j + w) * D) + c);
-                }
+                if (e < total) u[k] = __ldg(win + e);
             }
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
+            for (int k = 0; k < 8; ++k) {
                 const int e = b + k * blockDim.x;
                 if (e < total) s_buf[e] = u[k];
             }
         }
-        __syncthreads();
-        // pair p = (w, t): row w of the window against t = -1 (the entering
-        // reference) or the earlier window row t; pairs of row w start at w(w+1)/2
-        for (int p = warp; p < kPairs; p += kScanWarps) {
-            int w = 0;
-            while ((w + 1) * (w + 2) / 2 <= p) ++w;
-            const int t = p - w * (w + 1) / 2 - 1;
-            if (w >= nvalid) continue;
-            float dot, nv;
-            warp_dot(s_buf + (size_t)w * C, t < 0 ? ref : s_buf + (size_t)t * C, C, lane, t < 0,
-                     dot, nv);
-            if (lane == 0) {
-                s_dot[w][t + 1] = dot;
-                if (t < 0) s_nv[w] = nv;
-            }
+        if (threadIdx.x == 0) {
+            s_cur = -1;
+            s_w = 0;
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            int cur = -1;
-            float ncur = s_nr;
-            const int jr = s_jr;
-            for (int w = 0; w < nvalid; ++w) {
-                const float nv = s_nv[w];
-                float sim = 0.f;
-                if (nv > 0.f && ncur > 0.f)
-                    sim = __fdiv_rn(s_dot[w][cur + 1], __fmul_rn(__fsqrt_rn(nv), __fsqrt_rn(ncur)));
-                if (sim > tau) {
-                    src_pos[j + w] = cur < 0 ? jr : j + cur;
-                } else {
-                    src_pos[j + w] = j + w;
-                    cur = w;
-                    ncur = nv;
+        {
+            const int w = warp < kWin ? warp : warp - kWin;
+            const bool vs_ref = warp < kWin;
+            if (w < nvalid && (vs_ref || w > 0)) {
+                const uint4 *a = s_buf + (size_t)w * C;
+                float dot, nv;
+                warp_dot(a, vs_ref ? ref : a - C, C, lane, vs_ref, dot, nv);
+                if (lane == 0) {
+                    (vs_ref ? s_dref : s_dprev)[w] = dot;
+                    if (vs_ref) s_nv[w] = nv;
                 }
             }
-            s_newref = cur;
-            if (cur >= 0) {
-                s_jr = j + cur;
-                s_nr = ncur;
-            }
         }
-        __syncthreads();
-        const int nr = s_newref;
-        if (nr >= 0)
+        int have = -1;   // the row that s_dcur holds the similarities to
+        for (;;) {
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                int cur = s_cur, w = s_w;
+                const int jr = s_jr;
+                int more = 0;
+                for (; w < nvalid; ++w) {
+                    float dot;
+                    if (cur < 0) dot = s_dref[w];
+                    else if (cur == w - 1) dot = s_dprev[w];
+                    else if (cur == have) dot = s_dcur[w];
+                    else {
+                        more = 1;
+                        break;
+                    }
+                    const float nv = s_nv[w], ncur = cur < 0 ? s_nr : s_nv[cur];
+                    float sim = 0.f;
+                    if (nv > 0.f && ncur > 0.f)
+                        sim = __fdiv_rn(dot, __fmul_rn(__fsqrt_rn(nv), __fsqrt_rn(ncur)));
+                    if (sim > tau) {
+                        src_pos[j + w] = cur < 0 ? jr : j + cur;
+                    } else {
+                        src_pos[j + w] = j + w;
+                        cur = w;
+                    }
+                }
+                s_cur = cur;
+                s_w = w;
+                s_more = more;
+            }
+            __syncthreads();
+            if (!s_more) break;
+            const int cur = s_cur, w = s_w + warp;
+            if (w < nvalid) {
+                float dot, nv;
+                warp_dot(s_buf + (size_t)w * C, s_buf + (size_t)cur * C, C, lane, false, dot, nv);
+                if (lane == 0) s_dcur[w] = dot;
+            }
+            have = cur;
+        }
+        const int nr = s_cur;   // the last new reference carries into the next window
+        if (nr >= 0) {
+            if (threadIdx.x == 0) {
+                s_jr = j + nr;
+                s_nr = s_nv[nr];
+            }
             for (int c = threadIdx.x; c < C; c += blockDim.x) ref[c] = s_buf[(size_t)nr * C + c];
+        }
         __syncthreads();
     }
 }
