@@ -35,6 +35,7 @@ constexpr int BM = 128;        // queries per tile; two tiles per CTA
 constexpr int TILES = 2;
 constexpr int BN = 128;        // keys per block
 constexpr int RING_MAX = 8;    // K/V ring slots (K_j and V_j alternate)
+constexpr int PAIRS = 3;       // barriers of the pairs (V_j, K_{j+1}) in the ring
 constexpr int THREADS = 384;   // 4 control warps + 2 softmax warpgroups
 constexpr uint32_t TMEM_COLS = 512;   // S0, S1, O0, O1
 constexpr uint32_t O_COL = 256;
@@ -156,7 +157,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 
     // Every barrier is reused only after its previous phase has been observed
     // by its waiter, so no waiter can fall two phases behind.
-    __shared__ __align__(8) uint64_t q_full, ring_full[RING_MAX], ring_empty[RING_MAX];
+    __shared__ __align__(8) uint64_t q_full, pair_full[PAIRS], ring_empty[RING_MAX];
     __shared__ __align__(8) uint64_t s_full[TILES], p_full[TILES], pv_done[TILES];
     __shared__ __align__(8) uint64_t drain;
     __shared__ uint32_t tmem_slot;
@@ -173,7 +174,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 
     if (threadIdx.x == 0) {
         mbar_init(&q_full, 1);
-        for (int i = 0; i < RING; ++i) { mbar_init(&ring_full[i], 1); mbar_init(&ring_empty[i], 1); }
+        for (int i = 0; i < RING; ++i) mbar_init(&ring_empty[i], 1);
+        for (int i = 0; i < PAIRS; ++i) mbar_init(&pair_full[i], 1);
         for (int t = 0; t < TILES; ++t) {
             mbar_init(&s_full[t], 1);
             mbar_init(&p_full[t], 4);    // one arrival per softmax warp
@@ -199,27 +201,31 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     asm volatile("setmaxnreg.dec.sync.aligned.u32 48;" ::: "memory");
     if (warp == 0 && lane == 0) {
         // ---------------- TMA producer: Q0, Q1, then K_0, V_0, K_1, V_1, ... ----------------
+        // q_full covers both Q tiles and K_0, pair_full[j mod 3] covers V_j and K_{j+1}
         const int x0 = h * DH;
-        mbar_arrive_expect_tx(&q_full, TILES * C::Q_BYTES);
+        mbar_arrive_expect_tx(&q_full, TILES * C::Q_BYTES + C::SLOT_BYTES);
         for (int t = 0; t < TILES; ++t)
             for (int a = 0; a < C::ATOMS; ++a)
                 tma_load_2d(Qs + t * C::Q_BYTES + a * ATOM_BYTES, &tmQ, &q_full, x0 + 64 * a,
                             q0 + t * BM);
-        int issued = 0;
+        int armed = 0;
         for (int li = 0; li < 2 * nb; ++li) {
-            const int slot = li % RING;
+            const int slot = li % RING, pr = (li - 1) >> 1;
             if (!mbar_wait(&ring_empty[slot], ((li / RING) & 1) ^ 1, abort_v, p.err)) break;
-            mbar_arrive_expect_tx(&ring_full[slot], C::SLOT_BYTES);
+            uint64_t *full = li == 0 ? &q_full : &pair_full[pr % PAIRS];
+            if (li & 1) {   // V_j: arm the pair (the last one is V alone)
+                mbar_arrive_expect_tx(full, li + 1 < 2 * nb ? 2 * C::SLOT_BYTES : C::SLOT_BYTES);
+                armed = pr + 1;
+            }
             const CUtensorMap *m = (li & 1) ? &tmV : &tmK;
             for (int a = 0; a < C::ATOMS; ++a)
-                tma_load_2d(Ring + slot * C::SLOT_BYTES + a * ATOM_BYTES, m, &ring_full[slot],
-                            x0 + 64 * a, (kb0 + (li >> 1)) * BN);
-            issued = li + 1;
+                tma_load_2d(Ring + slot * C::SLOT_BYTES + a * ATOM_BYTES, m, full, x0 + 64 * a,
+                            (kb0 + (li >> 1)) * BN);
         }
         if (*abort_v) {  // let this CTA's copies land before it exits
             mbar_wait(&q_full, 0, abort_v, nullptr, 100000000ull);
-            for (int li = issued - RING < 0 ? 0 : issued - RING; li < issued; ++li)
-                mbar_wait(&ring_full[li % RING], (li / RING) & 1, abort_v, nullptr, 100000000ull);
+            for (int pr = armed - PAIRS < 0 ? 0 : armed - PAIRS; pr < armed; ++pr)
+                mbar_wait(&pair_full[pr % PAIRS], (pr / PAIRS) & 1, abort_v, nullptr, 100000000ull);
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
@@ -228,8 +234,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         // commits: the ring arithmetic and the descriptors then stay warp-uniform
         // and feed tcgen05.mma directly.  Issued from a single diverged lane, the
         // same loop ran the tensor cores about a quarter slower.
-        // Every wait and fence sits on the path that feeds the tensor cores:
-        // K_{j+1} is waited for before S0_{j+1}, V_{j+1} after S1_{j+1}.
+        // Every wait and fence sits on the path that feeds the tensor cores (about 130
+        // cycles each even when the phase has completed): V_j and K_{j+1} share a
+        // barrier, waited for once, in the window of tile 0's softmax.
         // P_t lives in the first 64 columns of S_t; S_t of the next block is
         // issued after P V of this block, and tcgen05.mma from one thread run in
         // order, so the S write cannot overtake the P read.  The commit of S_t
@@ -268,14 +275,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             for (int kk = 1; kk < BN / 16; ++kk)
                 tc_mma_f16_tmem_a(d, a + 8 * kk, desc(b_lo + (uint32_t)(kk * 2048 >> 4)), C::IDESC_PV, 1u);
         };
-        // ring position (slot, phase parity) of K_j; V_j is the next position
-        int ks = 0;
-        uint32_t kph = 0;
-        auto next = [&](int &slot, uint32_t &ph) { if (++slot == RING) { slot = 0; ph ^= 1u; } };
-        {   // K_0 and V_0, then S_0 of both tiles
-            int vs = ks; uint32_t vph = kph; next(vs, vph);
-            ok = ok && wait_all(&ring_full[ks], kph) && wait_all(&ring_full[vs], vph);
-        }
+        int ks = 0;                       // ring slot of K_j; V_j and K_{j+1} follow
+        int pr = 0;                       // barrier and parity of the pair (V_j, K_{j+1})
+        uint32_t pph = 0;
+        auto next_slot = [](int slot) { return slot + 1 == RING ? 0 : slot + 1; };
         if (ok) {
             tc_fence_after();
             if (leader) {
@@ -286,50 +289,44 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 tc_commit(&ring_empty[ks]);
             }
             __syncwarp();
+            ok = wait_all(&pair_full[0], 0);
         }
         for (int j = 0; ok && j < nb; ++j) {
-            int vs = ks; uint32_t vph = kph; next(vs, vph);       // V_j
-            int ns = vs; uint32_t nph = vph; next(ns, nph);       // K_{j+1}
-            int ws = ns; uint32_t wph = nph; next(ws, wph);       // V_{j+1}
+            const int vs = next_slot(ks), ns = next_slot(vs);     // V_j, K_{j+1}
             const bool more = j + 1 < nb;
             const uint32_t acc0 = j > 0 ? 1u : 0u;
-            // tile 0: P V_j, then S_{j+1} once K_{j+1} has landed
+            // tile 0: P V_j, then S_{j+1}
             if (!wait_all(&p_full[0], j & 1)) { ok = false; break; }
             tc_fence_after();
             if (leader) {
                 mma_pv(0, vs, acc0);
-                if (!more) tc_commit(&pv_done[0]);
-            }
-            __syncwarp();
-            if (more) {
-                if (!wait_all(&ring_full[ns], nph)) { ok = false; break; }
-                tc_fence_after();
-                if (leader) {
+                if (more) {
                     mma_s(0, ns);
                     tc_commit(&s_full[0]);
+                } else {
+                    tc_commit(&pv_done[0]);
                 }
-                __syncwarp();
             }
+            __syncwarp();
             // tile 1
             if (!wait_all(&p_full[1], j & 1)) { ok = false; break; }
             tc_fence_after();
             if (leader) {
                 mma_pv(1, vs, acc0);
                 tc_commit(&ring_empty[vs]);                      // V_j no longer needed
-                if (!more) tc_commit(&pv_done[1]);               // the last arrival of all
                 if (more) {
                     mma_s(1, ns);
                     tc_commit(&s_full[1]);
                     tc_commit(&ring_empty[ns]);                  // K_{j+1} no longer needed
+                } else {
+                    tc_commit(&pv_done[1]);                      // the last arrival of all
                 }
             }
             __syncwarp();
-            // V_{j+1} is read by the next block's P V only.  Waiting for it here
-            // rather than beside K_{j+1} puts the wait in the window in which
-            // tile 0's softmax forms P_{j+1}, and lets S0_{j+1} start sooner.
-            if (more && !wait_all(&ring_full[ws], wph)) { ok = false; break; }
+            // V_{j+1} and K_{j+2}: in the window in which tile 0's softmax forms P_{j+1}
+            if (++pr == PAIRS) { pr = 0; pph ^= 1u; }
+            if (more && !wait_all(&pair_full[pr], pph)) { ok = false; break; }
             ks = ns;
-            kph = nph;
         }
         if (!ok && leader) {  // wait for the MMAs already issued before tensor memory is freed
             tc_commit(&drain);
