@@ -9,7 +9,9 @@
 // topk_kernel: one CTA radix-selects the K-th largest 32-bit key (11/11/10-bit
 //   digits), then compacts in index order, taking keys equal to the threshold
 //   from the lowest index up.  Keys are read four at a time (16-byte loads,
-//   several in flight per thread): the kernel is bound by load latency.
+//   several in flight per thread): the kernel is bound by load latency and block
+//   barriers.  A digit is looked up with one barrier and a tile of 8192 keys is
+//   compacted with one (five and six before): 7800 keys 10.6 -> 9.2 us.
 // topk_cluster_kernel: the same selection with the keys split over a cluster
 //   of 8 CTAs, the histograms summed through distributed shared memory; used
 //   from 10240 keys up (28.7 -> 18.3 us at 32760 keys, 53 -> 20 us at 63960).
@@ -23,7 +25,9 @@ namespace {
 constexpr int kDriftThreads = 256;
 constexpr int kDriftUnroll = 4;
 constexpr int kTopkThreads = 1024;
-constexpr int kTopkItems = 4;
+constexpr int kTopkItems = 8;
+constexpr int kTopkKeyBytesMax = 200 * 1024;   // keys of one CTA in shared memory
+constexpr int kTopkSliceMax = kTopkKeyBytesMax / 4;
 
 ECHO_DEV float segment_weight(float e, float emax, float lam) {
     if (!(emax > 0.f)) return 1.f;
@@ -167,34 +171,28 @@ ECHO_DEV uint32_t order_key(float f) {
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
-// Exclusive block scan of one value per thread (blockDim == kTopkThreads).
-// Returns the exclusive prefix; *total gets the block sum.
-ECHO_DEV int block_exclusive_scan(int v, int *warp_sums, int *total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int inc = v;
+ECHO_DEV uint32_t warp_inclusive_scan(uint32_t v) {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const int n = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += n;
+        const uint32_t n = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += n;
     }
+    return v;
+}
+
+// Exclusive block scan of one value per thread (blockDim == kTopkThreads = 32 warps).
+// Returns the exclusive prefix; *total gets the block sum.  One block barrier: every
+// warp scans the 32 warp sums for itself.  Consecutive calls take different
+// `warp_sums` (32 words).
+ECHO_DEV uint32_t block_exclusive_scan(uint32_t v, uint32_t *warp_sums, uint32_t *total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t inc = warp_inclusive_scan(v);
     if (lane == 31) warp_sums[warp] = inc;
     __syncthreads();
-    if (warp == 0) {
-        int w = warp_sums[lane];
-        int wi = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int n = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += n;
-        }
-        warp_sums[lane] = wi - w;           // exclusive prefix of warp totals
-        if (lane == 31) warp_sums[32] = wi; // block total
-    }
-    __syncthreads();
-    const int r = warp_sums[warp] + inc - v;
-    *total = warp_sums[32];
-    __syncthreads();
-    return r;
+    const uint32_t t = warp_sums[lane], ti = warp_inclusive_scan(t);
+    *total = __shfl_sync(0xffffffffu, ti, 31);
+    return __shfl_sync(0xffffffffu, ti - t, warp) + inc - v;
 }
 
 // Radix digits (bits [sh, sh + log2 nb)) of the n keys whose higher bits
@@ -224,76 +222,75 @@ ECHO_DEV void count_digits(KeyFn keys4, int n, int sh, int nb, uint32_t prefix, 
     }
 }
 
-// The digit that holds the krem-th largest counted key, the bins taken from
-// the highest down (thread t covers hi = nb-1-2t and hi-1); krem becomes that
-// key's rank within its bin.  Every thread returns the same digit.
-ECHO_DEV int pick_digit(const int *hist, int nb, int &krem, int *warp_sums, int *s_digit,
-                        int *s_krem) {
-    const int hi = nb - 1 - 2 * (int)threadIdx.x;
-    const int c_hi = hi >= 0 ? hist[hi] : 0;
-    const int c_lo = hi - 1 >= 0 ? hist[hi - 1] : 0;
-    int total;
-    const int above = block_exclusive_scan(c_hi + c_lo, warp_sums, &total);
-    if (hi >= 0 && above < krem && above + c_hi >= krem) {
-        *s_digit = hi;
-        *s_krem = krem - above;
-    }
-    if (hi - 1 >= 0 && above + c_hi < krem && above + c_hi + c_lo >= krem) {
-        *s_digit = hi - 1;
-        *s_krem = krem - above - c_hi;
-    }
+// The digit that holds the krem-th largest counted key, the bins taken from the
+// highest down; krem becomes that key's rank within its bin.  Every thread returns
+// the same digit.  Warp g sums the g-th 32nd of the bins; after one block barrier
+// every warp looks up the 32nd and then the bin for itself.  `sums`: 32 words, not
+// those of the call before.
+ECHO_DEV int pick_digit(const int *hist, int nb, int &krem, uint32_t *sums) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int per = nb >> 10;                      // bins per lane: 2 (2048) or 1 (1024)
+    auto bins = [&](int g, int &c0, int &c1) {     // lane's bins of the g-th 32nd, descending
+        const int top = nb - 1 - (g * 32 + lane) * per;
+        c0 = hist[top];
+        c1 = per == 2 ? hist[top - 1] : 0;
+        return top;
+    };
+    int c0, c1;
+    bins(warp, c0, c1);
+    const uint32_t mine = __reduce_add_sync(0xffffffffu, (uint32_t)(c0 + c1));
+    if (lane == 0) sums[warp] = mine;
     __syncthreads();
-    const int digit = *s_digit;
-    krem = *s_krem;
-    __syncthreads();
-    return digit;
+    const uint32_t t = sums[lane], ti = warp_inclusive_scan(t);
+    const int g = __ffs(__ballot_sync(0xffffffffu, ti >= (uint32_t)krem)) - 1;
+    const int above = (int)__shfl_sync(0xffffffffu, ti - t, g);
+    const int top = bins(g, c0, c1);
+    const int before = above + (int)warp_inclusive_scan((uint32_t)(c0 + c1)) - c0 - c1;
+    const int l = __ffs(__ballot_sync(0xffffffffu, before + c0 + c1 >= krem)) - 1;
+    const bool second = before + c0 < krem;        // the lower of the lane's two bins
+    krem = __shfl_sync(0xffffffffu, krem - before - (second ? c0 : 0), l);
+    return __shfl_sync(0xffffffffu, second ? top - 1 : top, l);
 }
 
 // Writes, in index order, the indices (first + i) of the n keys above thr and
 // of the keys equal to thr while fewer than need_eq of those have been taken.
 // eq_run and sel_run: keys equal to thr and keys taken before key 0 (by
-// lower-ranked slices); the first index written goes to idx[sel_run].
+// lower-ranked slices); the first index written goes to idx[sel_run].  One block
+// scan per tile carries both counts (above in the low half, equal in the high).
 template <typename KeyFn>
 ECHO_DEV void compact_in_index_order(KeyFn keys4, int n, int first, uint32_t thr, int need_eq,
                                      int eq_run, int sel_run, int32_t *__restrict__ idx,
-                                     int *warp_sums) {
-    const int tile = kTopkThreads * kTopkItems;
-    for (int base = 0; base < n; base += tile) {
-        bool gt[kTopkItems], eq[kTopkItems];
-        int neq = 0;
+                                     uint32_t (*warp_sums)[32]) {
+    constexpr int tile = kTopkThreads * kTopkItems;
+    static_assert(tile < 65536, "a tile's counts fit 16 bits");
+    int turn = 0;
+    for (int base = 0; base < n; base += tile, turn ^= 1) {
         const int i0 = base + (int)threadIdx.x * kTopkItems;
-        const uint4 kv4 = i0 < n ? keys4(i0) : make_uint4(0, 0, 0, 0);
-        const uint32_t kk[4] = {kv4.x, kv4.y, kv4.z, kv4.w};
+        uint32_t kk[kTopkItems];
 #pragma unroll
-        for (int j = 0; j < kTopkItems; ++j) {
-            const int i = i0 + j;
-            gt[j] = eq[j] = false;
-            if (i < n) {
-                gt[j] = kk[j] > thr;
-                eq[j] = kk[j] == thr;
-            }
-            neq += eq[j];
+        for (int j = 0; j < kTopkItems; j += 4) {
+            const uint4 v = i0 + j < n ? keys4(i0 + j) : make_uint4(0, 0, 0, 0);
+            kk[j] = v.x; kk[j + 1] = v.y; kk[j + 2] = v.z; kk[j + 3] = v.w;
         }
-        int eq_total;
-        int eq_before = eq_run + block_exclusive_scan(neq, warp_sums, &eq_total);
-        bool sel[kTopkItems];
-        int nsel = 0;
-#pragma unroll
-        for (int j = 0; j < kTopkItems; ++j) {
-            sel[j] = gt[j];
-            if (eq[j]) {
-                sel[j] = eq_before < need_eq;
-                ++eq_before;
-            }
-            nsel += sel[j];
-        }
-        int sel_total;
-        int pos = sel_run + block_exclusive_scan(nsel, warp_sums, &sel_total);
+        uint32_t cnt = 0;
 #pragma unroll
         for (int j = 0; j < kTopkItems; ++j)
-            if (sel[j]) idx[pos++] = first + i0 + j;
-        eq_run += eq_total;
-        sel_run += sel_total;
+            if (i0 + j < n) cnt += (uint32_t)(kk[j] > thr) + ((uint32_t)(kk[j] == thr) << 16);
+        uint32_t tot;
+        const uint32_t pre = block_exclusive_scan(cnt, warp_sums[turn], &tot);
+        int eq = eq_run + (int)(pre >> 16);
+        const int eq_taken0 = min(eq_run, need_eq);
+        int pos = sel_run + (int)(pre & 0xffffu) + min(eq, need_eq) - eq_taken0;
+#pragma unroll
+        for (int j = 0; j < kTopkItems; ++j) {
+            if (i0 + j >= n) break;
+            bool sel = kk[j] > thr;
+            if (kk[j] == thr) sel = eq++ < need_eq;
+            if (sel) idx[pos++] = first + i0 + j;
+        }
+        sel_run += (int)(tot & 0xffffu) - eq_taken0;
+        eq_run += (int)(tot >> 16);
+        sel_run += min(eq_run, need_eq);
     }
 }
 
@@ -302,9 +299,8 @@ topk_kernel(const float *__restrict__ scores, int NT, int K, int keys_in_smem,
             int32_t *__restrict__ idx) {
     pdl_enter();
     extern __shared__ uint32_t skeys[];
-    __shared__ int hist[2048];
-    __shared__ int warp_sums[33];
-    __shared__ int s_digit, s_krem;
+    __shared__ int hist[3][2048];          // one per pass, cleared together
+    __shared__ uint32_t sums[5][32];       // a block scan's or look-up's warp sums
     const int tid = threadIdx.x;
 
     if (K >= NT) {
@@ -325,6 +321,7 @@ topk_kernel(const float *__restrict__ scores, int NT, int K, int keys_in_smem,
         for (int c = 0; c < 4; ++c) k[c] = i + c < NT ? order_key(scores[i + c]) : 0u;
         return make_uint4(k[0], k[1], k[2], k[3]);
     };
+    for (int b = tid; b < 3 * 2048; b += blockDim.x) (&hist[0][0])[b] = 0;
     const int stride4 = blockDim.x * 4;
     if (keys_in_smem) {
         // eight 16-byte loads in flight per thread
@@ -354,16 +351,14 @@ topk_kernel(const float *__restrict__ scores, int NT, int K, int keys_in_smem,
     for (int pass = 0; pass < 3; ++pass) {
         const int sh = shifts[pass];
         const int nb = 1 << widths[pass];
-        for (int b = tid; b < 2048; b += blockDim.x) hist[b] = 0;
+        count_digits(keys4, NT, sh, nb, prefix, pmask, hist[pass]);
         __syncthreads();
-        count_digits(keys4, NT, sh, nb, prefix, pmask, hist);
-        __syncthreads();
-        prefix |= (uint32_t)pick_digit(hist, nb, krem, warp_sums, &s_digit, &s_krem) << sh;
+        prefix |= (uint32_t)pick_digit(hist[pass], nb, krem, sums[pass]) << sh;
         pmask |= (uint32_t)(nb - 1) << sh;
     }
     // prefix is the K-th largest key; take every larger key and the first
     // `krem` keys equal to it in index order.
-    compact_in_index_order(keys4, NT, 0, prefix, krem, 0, 0, idx, warp_sums);
+    compact_in_index_order(keys4, NT, 0, prefix, krem, 0, 0, idx, sums + 3);
 }
 
 constexpr int kTopkClusterCtas = 8;
@@ -403,8 +398,7 @@ topk_cluster_kernel(const float *__restrict__ scores, int NT, int K, int slice,
     __shared__ __align__(16) int hist[2048];                  // this CTA's counts
     __shared__ __align__(16) int red[3][kBinsPerRank];        // owned bins, one buffer a pass
     __shared__ __align__(16) int full[2048];                  // the cluster's counts
-    __shared__ int warp_sums[33];
-    __shared__ int s_digit, s_krem;
+    __shared__ uint32_t sums[6][32];       // a block scan's or look-up's warp sums
     __shared__ int s_counts[2];   // keys of this slice above / equal to the threshold
     const int tid = threadIdx.x;
     const int rank = (int)cluster_ctarank();
@@ -471,30 +465,26 @@ topk_cluster_kernel(const float *__restrict__ scores, int NT, int K, int slice,
             *reinterpret_cast<int4 *>(&full[b0]) = v;
         }
         __syncthreads();
-        prefix |= (uint32_t)pick_digit(full, nb, krem, warp_sums, &s_digit, &s_krem) << sh;
+        prefix |= (uint32_t)pick_digit(full, nb, krem, sums[pass]) << sh;
         pmask |= (uint32_t)(nb - 1) << sh;
     }
     const uint32_t thr = prefix;
     const int need_eq = krem;
 
-    // this slice's counts above / equal to the threshold
-    int n_gt = 0, n_eq = 0;
+    // this slice's counts above (low half) / equal to (high half) the threshold
+    static_assert(kTopkSliceMax < 65536, "a slice's counts fit 16 bits");
+    uint32_t cnt = 0, cnt_total;
     for (int b = tid * 4; b < n; b += stride4) {
         const uint4 v = skeys4[b >> 2];
         const uint32_t k[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int c = 0; c < 4; ++c)
-            if (b + c < n) {
-                n_gt += k[c] > thr;
-                n_eq += k[c] == thr;
-            }
+            if (b + c < n) cnt += (uint32_t)(k[c] > thr) + ((uint32_t)(k[c] == thr) << 16);
     }
-    int gt_total, eq_total_slice;
-    block_exclusive_scan(n_gt, warp_sums, &gt_total);
-    block_exclusive_scan(n_eq, warp_sums, &eq_total_slice);
+    block_exclusive_scan(cnt, sums[3], &cnt_total);
     if (tid == 0) {
-        s_counts[0] = gt_total;
-        s_counts[1] = eq_total_slice;
+        s_counts[0] = (int)(cnt_total & 0xffffu);
+        s_counts[1] = (int)(cnt_total >> 16);
     }
     cluster_sync_all();
     int gt_before = 0, eq_before = 0;
@@ -503,12 +493,10 @@ topk_cluster_kernel(const float *__restrict__ scores, int NT, int K, int slice,
         eq_before += ld_shared_cluster_s32(mapa_shared(smem_u32(&s_counts[1]), (uint32_t)r));
     }
     compact_in_index_order(keys4, n, lo, thr, need_eq, eq_before,
-                           gt_before + min(eq_before, need_eq), idx, warp_sums);
+                           gt_before + min(eq_before, need_eq), idx, sums + 4);
     cluster_sync_all();   // no CTA leaves while another may still read its counts
 }
 
-constexpr int kTopkKeyBytesMax = 200 * 1024;   // keys of one CTA in shared memory
-constexpr int kTopkSliceMax = kTopkKeyBytesMax / 4;
 constexpr int kTopkClusterMinKeys = 10240;   // below: the one-CTA kernel is faster
 
 // Both top-K kernels may take up to kTopkKeyBytesMax of dynamic shared memory
