@@ -161,7 +161,7 @@ echo_status run_active(const echo_block_weights *w, const echo_block_dims &d, co
     echo_status s = ECHO_OK;
     // the row map, and max |y_act| per row cleared for the FFN-down epilogue
     uint32_t *amax = reinterpret_cast<uint32_t *>(ws + L.amax);
-    launch_rowmap(idx, K, NT, rowmap, amax, K, st);
+    if (K <= 0 || n_kv_rows >= 0) launch_rowmap(idx, K, NT, rowmap, amax, K, st);
     if (K > 0) {
         // Q' and the K/V that are not there yet in one launch: alone, the few tiles of
         // Q' would leave most SM pairs idle (7800 tokens, D 1024, K 1560: 36 -> 29 us)
@@ -175,7 +175,7 @@ echo_status run_active(const echo_block_weights *w, const echo_block_dims &d, co
             s = launch_linear_pair(kvproj, qproj, st);
         } else {
             // LN over every latent; the active rows also land in na, gathered
-            launch_layernorm_scatter(x, NT, D, n1, rowmap, na, st);
+            launch_layernorm_active(x, NT, D, n1, idx, K, rowmap, amax, na, st);
             s = launch_linear_pair({n1, D, NT, D, w->Wkv, w->bkv, 2 * D, 0, nullptr, ECHO_BF16,
                                     nullptr, kv, 2 * (int64_t)D, ECHO_BF16}, qproj, st);
         }

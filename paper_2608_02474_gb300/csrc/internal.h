@@ -76,9 +76,12 @@ bool make_tmap_bf16(CUtensorMap *m, const void *base, uint64_t rows, uint64_t co
 // layernorm.cu
 void launch_layernorm(const void *in, echo_dtype in_t, const int32_t *rows, int32_t n_rows,
                       int32_t D, void *out, cudaStream_t st);
-// out = LN(in) for all n_rows bf16 rows; row i also goes to out2[map[i]] when map[i] >= 0
-void launch_layernorm_scatter(const void *in, int32_t n_rows, int32_t D, void *out,
-                              const int32_t *scatter_map, void *out2, cudaStream_t st);
+// out = LN(in) for all n_rows bf16 rows; rowmap as launch_rowmap makes it from idx[0 .. K),
+// K > 0, with zero[0 .. K) cleared; row i also goes to out2[rowmap[i]] when that is >= 0.
+// Up to D = 2048 one launch: each row's warp looks it up in idx itself, while the row is
+// on its way (four layers of 7800 tokens, D 1024: 837 -> 826 us a step).
+void launch_layernorm_active(const void *in, int32_t n_rows, int32_t D, void *out, const int32_t *idx,
+                             int32_t K, int32_t *rowmap, uint32_t *zero, void *out2, cudaStream_t st);
 
 // gemm.cu: out = act(A W^T + bias) + resid
 struct LinearArgs {

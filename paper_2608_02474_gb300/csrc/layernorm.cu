@@ -113,14 +113,34 @@ layernorm_kernel(const T *__restrict__ in, const int32_t *__restrict__ rows, int
     }
 }
 
+// position of v in idx[0 .. n) (ascending, distinct), or -1: 32 probes at a time
+ECHO_DEV int warp_find(const int32_t *__restrict__ idx, int n, int v) {
+    const int lane = threadIdx.x & 31;
+    int lo = 0;
+    while (n > 0) {
+        const int step = (n + 31) >> 5;   // each lane looks at the first of `step` entries
+        const int x = lane * step < n ? idx[lo + lane * step] : INT32_MAX;
+        const uint32_t le = __ballot_sync(0xffffffffu, x <= v);
+        if (!le) return -1;
+        const int b = 31 - __clz((int)le);
+        lo += b * step;
+        n = min(step, n - b * step);
+        if (n == 1) return __shfl_sync(0xffffffffu, x, b) == v ? lo : -1;
+    }
+    return -1;
+}
+
 // bf16 input: one warp per row, the row held packed in registers (CPL 16-byte
 // chunks per lane), so each row is read from HBM once and no block barrier is
-// needed.  scatter_map and out2 as in layernorm_bulk_bf16.
+// needed.  With idx (ascending, distinct), row j is also looked up there: its
+// position p (-1: not in it) goes to rowmap[j], zero[p] is cleared, and the result
+// is written to out2[p] as well.
 template <int CPL>
 __global__ void __launch_bounds__(kThreads)
 layernorm_warp_bf16(const __nv_bfloat16 *__restrict__ in, const int32_t *__restrict__ rows,
-                    int n_rows, int D, __nv_bfloat16 *__restrict__ out,
-                    const int32_t *__restrict__ scatter_map, __nv_bfloat16 *__restrict__ out2) {
+                    int n_rows, int D, __nv_bfloat16 *__restrict__ out, __nv_bfloat16 *__restrict__ out2,
+                    const int32_t *__restrict__ idx, int n_idx, int32_t *__restrict__ rowmap,
+                    uint32_t *__restrict__ zero) {
     pdl_enter();
     const int lane = threadIdx.x & 31;
     const int warps = kThreads / 32;
@@ -128,13 +148,20 @@ layernorm_warp_bf16(const __nv_bfloat16 *__restrict__ in, const int32_t *__restr
     const float invD = 1.f / (float)D;
     for (int j = blockIdx.x * warps + (threadIdx.x >> 5); j < n_rows; j += gridDim.x * warps) {
         const int r = rows ? rows[j] : j;
-        const int j2 = scatter_map ? scatter_map[j] : -1;
         const uint4 *src = reinterpret_cast<const uint4 *>(in + (int64_t)r * D);
         uint4 v[CPL];
 #pragma unroll
         for (int k = 0; k < CPL; ++k) {
             const int c = lane + 32 * k;
             v[k] = c < C ? __ldcs(src + c) : make_uint4(0, 0, 0, 0);
+        }
+        int j2 = -1;
+        if (idx) {   // while the row is on its way
+            j2 = warp_find(idx, n_idx, j);
+            if (lane == 0) {
+                rowmap[j] = j2;
+                if (j2 >= 0) zero[j2] = 0u;
+            }
         }
         float s = 0.f;
 #pragma unroll
@@ -311,26 +338,28 @@ void launch_bulk_bf16(const __nv_bfloat16 *in, int n_rows, int D, __nv_bfloat16 
 
 template <int CPL>
 void launch_warp_bf16(const __nv_bfloat16 *in, const int32_t *rows, int n_rows, int D,
-                      __nv_bfloat16 *out, const int32_t *scatter_map, __nv_bfloat16 *out2,
-                      cudaStream_t st) {
+                      __nv_bfloat16 *out, __nv_bfloat16 *out2, const int32_t *idx, int n_idx,
+                      int32_t *rowmap, uint32_t *zero, cudaStream_t st) {
     constexpr int RPB = kThreads / 32;
     int grid = (n_rows + RPB - 1) / RPB;
     if (grid > 152 * 8) grid = 152 * 8;
     echo::launch_chained(layernorm_warp_bf16<CPL>, dim3(grid), dim3(kThreads), 0, st, in, rows,
-                         n_rows, D, out, scatter_map, out2);
+                         n_rows, D, out, out2, idx, n_idx, rowmap, zero);
 }
 
 // the row packed in registers: gathered rows, and every row up to D = kWarpRowMax
 void launch_regs_bf16(const __nv_bfloat16 *in, const int32_t *rows, int n_rows, int D,
-                      __nv_bfloat16 *out, const int32_t *map, __nv_bfloat16 *out2, cudaStream_t st) {
+                      __nv_bfloat16 *out, __nv_bfloat16 *out2, const int32_t *idx, int n_idx,
+                      int32_t *rowmap, uint32_t *zero, cudaStream_t st) {
     const int cpl = (D / 8 + 31) / 32;   // 16-byte chunks per lane
-    if (cpl <= 1) return launch_warp_bf16<1>(in, rows, n_rows, D, out, map, out2, st);
-    if (cpl <= 4) return launch_warp_bf16<4>(in, rows, n_rows, D, out, map, out2, st);
-    if (cpl <= 8) return launch_warp_bf16<8>(in, rows, n_rows, D, out, map, out2, st);
-    if (cpl <= 16) return launch_warp_bf16<16>(in, rows, n_rows, D, out, map, out2, st);
-    if (cpl <= 20) return launch_warp_bf16<20>(in, rows, n_rows, D, out, map, out2, st);
-    if (cpl <= 24) return launch_warp_bf16<24>(in, rows, n_rows, D, out, map, out2, st);
-    return launch_warp_bf16<32>(in, rows, n_rows, D, out, map, out2, st);
+    auto go = [&](auto launch) { launch(in, rows, n_rows, D, out, out2, idx, n_idx, rowmap, zero, st); };
+    if (cpl <= 1) return go(launch_warp_bf16<1>);
+    if (cpl <= 4) return go(launch_warp_bf16<4>);
+    if (cpl <= 8) return go(launch_warp_bf16<8>);
+    if (cpl <= 16) return go(launch_warp_bf16<16>);
+    if (cpl <= 20) return go(launch_warp_bf16<20>);
+    if (cpl <= 24) return go(launch_warp_bf16<24>);
+    return go(launch_warp_bf16<32>);
 }
 
 // fp32 rows of up to kWarpRowMax values: one warp per row, the row in registers
@@ -453,8 +482,8 @@ void launch_all_f32(const float *in, int n_rows, int D, __nv_bfloat16 *out, cuda
 // bulk-copy kernel (the same arithmetic as layernorm_warp_bf16)
 void launch_all_bf16(const __nv_bfloat16 *in, int n_rows, int D, __nv_bfloat16 *out,
                      const int32_t *scatter_map, __nv_bfloat16 *out2, cudaStream_t st) {
-    if (D <= kWarpRowMax)
-        return launch_regs_bf16(in, nullptr, n_rows, D, out, scatter_map, out2, st);
+    if (D <= kWarpRowMax && !scatter_map)
+        return launch_regs_bf16(in, nullptr, n_rows, D, out, nullptr, nullptr, 0, nullptr, nullptr, st);
     const int cpl = (D / 8 + 31) / 32;
     if (cpl <= 16) return launch_bulk_bf16<16>(in, n_rows, D, out, scatter_map, out2, st);
     if (cpl <= 20) return launch_bulk_bf16<20>(in, n_rows, D, out, scatter_map, out2, st);
@@ -469,7 +498,7 @@ void launch_t(const T *in, const int32_t *rows, int n_rows, int D, __nv_bfloat16
     echo::LaunchScope ls(ECHO_K_LAYERNORM, n_rows, D, (int64_t)sizeof(T), st);
     if constexpr (sizeof(T) == 2) {
         if (!rows) return launch_all_bf16(in, n_rows, D, out, nullptr, nullptr, st);
-        return launch_regs_bf16(in, rows, n_rows, D, out, nullptr, nullptr, st);
+        return launch_regs_bf16(in, rows, n_rows, D, out, nullptr, nullptr, 0, nullptr, nullptr, st);
     } else {
         if (!rows) return launch_all_f32(in, n_rows, D, out, st);
     }
@@ -492,13 +521,19 @@ void launch_t(const T *in, const int32_t *rows, int n_rows, int D, __nv_bfloat16
 
 namespace echo {
 
-void launch_layernorm_scatter(const void *in, int32_t n_rows, int32_t D, void *out,
-                              const int32_t *scatter_map, void *out2, cudaStream_t st) {
+void launch_layernorm_active(const void *in, int32_t n_rows, int32_t D, void *out, const int32_t *idx,
+                             int32_t K, int32_t *rowmap, uint32_t *zero, void *out2,
+                             cudaStream_t st) {
     if (n_rows <= 0) return;
+    const __nv_bfloat16 *x = static_cast<const __nv_bfloat16 *>(in);
+    __nv_bfloat16 *o = static_cast<__nv_bfloat16 *>(out), *o2 = static_cast<__nv_bfloat16 *>(out2);
+    if (D <= kWarpRowMax) {
+        LaunchScope ls(ECHO_K_LAYERNORM, n_rows, D, 2, st);
+        return launch_regs_bf16(x, nullptr, n_rows, D, o, o2, idx, K, rowmap, zero, st);
+    }
+    launch_rowmap(idx, K, n_rows, rowmap, zero, K, st);
     LaunchScope ls(ECHO_K_LAYERNORM, n_rows, D, 2, st);
-    launch_all_bf16(static_cast<const __nv_bfloat16 *>(in), n_rows, D,
-                    static_cast<__nv_bfloat16 *>(out), scatter_map,
-                    static_cast<__nv_bfloat16 *>(out2), st);
+    launch_all_bf16(x, n_rows, D, o, rowmap, o2, st);
 }
 
 void launch_layernorm(const void *in, echo_dtype in_t, const int32_t *rows, int32_t n_rows,
