@@ -59,6 +59,7 @@ struct Cfg {
 
 struct AttnParams {
     int M, L;
+    int ntp, item0;   // tile pairs of a head; the grid's first (tile pair, head)
     float scale_log2;
     __nv_bfloat16 *O;
     int64_t ldo;
@@ -164,10 +165,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     __shared__ int abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int h = blockIdx.y;
     // the CTAs of a cluster share the queries and split the key blocks
     const int splits = SPLIT ? (int)cluster_nctarank() : 1, split = SPLIT ? (int)cluster_ctarank() : 0;
-    const int q0 = ((int)blockIdx.x / splits) * (TILES * BM);
+    const int item = p.item0 + (int)blockIdx.x / splits;
+    const int h = item / p.ntp, q0 = (item - h * p.ntp) * (TILES * BM);
     const int nb_all = (p.L + BN - 1) / BN;
     const int kb0 = SPLIT ? (int)((int64_t)nb_all * split / splits) : 0;   // this CTA's first block
     const int nb = SPLIT ? (int)((int64_t)nb_all * (split + 1) / splits) - kb0 : nb_all;
@@ -540,10 +541,10 @@ attn_d64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     __shared__ int abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int h = blockIdx.y;
     // the CTAs of a cluster share the queries and split the key blocks
     const int splits = SPLIT ? (int)cluster_nctarank() : 1, split = SPLIT ? (int)cluster_ctarank() : 0;
-    const int q0 = ((int)blockIdx.x / splits) * (TILES * BM);
+    const int item = p.item0 + (int)blockIdx.x / splits;
+    const int h = item / p.ntp, q0 = (item - h * p.ntp) * (TILES * BM);
     const int nb_all = (p.L + BN - 1) / BN;
     const int kb0 = SPLIT ? (int)((int64_t)nb_all * split / splits) : 0;   // this CTA's first block
     const int nb = SPLIT ? (int)((int64_t)nb_all * (split + 1) / splits) - kb0 : nb_all;
@@ -1371,6 +1372,7 @@ echo_status launch_items_dh(const void *Q, int64_t ldq, const void *K, const voi
 }
 
 constexpr int kSplitMax = 8;   // CTAs of a cluster (portable size)
+constexpr int kTailFixed = 4;  // a second launch, in the key-block times of choose_splits
 
 // the one-shot kernel of a head size
 template <int DH, bool SPLIT>
@@ -1435,14 +1437,13 @@ int split_slots(int splits) {
 // (set-up and epilogue 4; with the sum over the cluster 7).  Measured, one CTA
 // against the split chosen: 389 queries x 7801 keys, 16 heads of 64: 61 -> 23 us
 // (4); 130 x 2000 x 6 heads of 64: 21.4 -> 10.2 us (8); 600 x 2000 x 16 heads of
-// 64: 22.0 -> 14.1 us (2); 3198 x 63960 x 40 heads of 128 (3.4 waves): 2.71 ->
-// 2.60 ms under the power cap (2).  At 1560 x 7800 x 16 (0.74 waves) two take
+// 64: 22.0 -> 14.1 us (2).  At 1560 x 7800 x 16 (0.74 waves) two take
 // 72 us against 62 and the rule stays at one.
 template <int DH>
-int choose_splits(int64_t items, int nb) {
-    int best = 1;
-    int64_t best_cost = INT64_MAX;
-    for (int sp = 1; sp <= kSplitMax && sp <= nb; sp *= 2) {
+int choose_splits(int64_t items, int nb, int least, int64_t &best_cost) {
+    int best = 0;
+    best_cost = INT64_MAX;
+    for (int sp = least; sp <= kSplitMax && sp <= nb; sp *= 2) {
         const int slots = split_slots<DH>(sp);
         if (!slots) continue;
         const int64_t waves = (items * sp + slots - 1) / slots;
@@ -1452,9 +1453,36 @@ int choose_splits(int64_t items, int nb) {
     return best;
 }
 
+// Items that are neither one wave nor many leave a last wave with few CTAs that
+// each walk every key.  The whole waves then run on one CTA per item, and the
+// items left over in a second launch with their keys split, where the sum of both
+// is less than one launch of either form.  (kTailFixed: the first launch's CTAs
+// end at different times, and the second waits for the last.)  Measured, one
+// launch against two: 7800 x 7800 x 16 heads of 64 (3.3 waves) 244 -> 226 us;
+// 2600 x 7800 x 16 (1.2) 131 -> 103; 5000 x 4000 x 8 (1.1) 70 -> 51; 1300 x 30000 x 40
+// (1.6) 471 -> 435; heads of 128: 2600 x 2200 x 16 (1.2) 54 -> 45, 1700 x 12000 x 32
+// (1.5) 210 -> 198, 4000 x 4000 x 24 (2.5) 137 -> 133.  Below 2049 keys the
+// persistent kernel has no such waves.
+struct Plan {
+    int64_t whole;   // the first items: one CTA each
+    int splits;      // CTAs of each of the others
+};
+
+template <int DH>
+Plan choose_plan(int64_t items, int nb, int L) {
+    int64_t cost, tail_cost;
+    const int splits = choose_splits<DH>(items, nb, 1, cost);
+    const int64_t waves = items / num_sms(), whole = waves * num_sms();
+    if (L > kItemsMaxKeys && whole > 0 && whole < items) {
+        const int tail = choose_splits<DH>(items - whole, nb, 2, tail_cost);
+        if (tail && waves * (nb + 4) + tail_cost + kTailFixed < cost) return {whole, tail};
+    }
+    return splits > 1 ? Plan{0, splits} : Plan{items, 1};
+}
+
 template <int DH>
 echo_status launch_dh(const void *Q, int64_t ldq, const void *K, const void *V, int64_t ldkv, int M,
-                      int L, int H, int splits, void *O, int64_t ldo, cudaStream_t st) {
+                      int L, int H, Plan plan, void *O, int64_t ldo, cudaStream_t st) {
     raise_smem_cap<DH>();
     CUtensorMap tq, tk, tv;
     const uint64_t cols = (uint64_t)H * DH;
@@ -1469,16 +1497,17 @@ echo_status launch_dh(const void *Q, int64_t ldq, const void *K, const void *V, 
     p.O = static_cast<__nv_bfloat16 *>(O);
     p.ldo = ldo;
     p.err = echo::device_error_ptr();
-    const int ntp = (M + TILES * BM - 1) / (TILES * BM);
-    if (splits == 1) {
-        echo::LaunchScope ls(ECHO_K_ATTENTION, M, L, (int64_t)H * DH, st);
-        echo::launch_chained(one_shot_kernel<DH, false>(), dim3(ntp, H), dim3(one_shot_threads<DH>()),
-                             one_shot_smem<DH>(), st, tq, tk, tv, p);
-        return echo::last_launch_status();
-    }
+    p.ntp = (M + TILES * BM - 1) / (TILES * BM);
+    p.item0 = 0;
+    const int64_t rest = (int64_t)p.ntp * H - plan.whole;
     echo::LaunchScope ls(ECHO_K_ATTENTION, M, L, (int64_t)H * DH, st);
-    if (echo::launch_chained_cluster((unsigned)splits, one_shot_kernel<DH, true>(),
-                                     dim3((unsigned)(ntp * splits), (unsigned)H),
+    if (plan.whole > 0)
+        echo::launch_chained(one_shot_kernel<DH, false>(), dim3((unsigned)plan.whole),
+                             dim3(one_shot_threads<DH>()), one_shot_smem<DH>(), st, tq, tk, tv, p);
+    p.item0 = (int)plan.whole;
+    if (rest > 0 &&
+        echo::launch_chained_cluster((unsigned)plan.splits, one_shot_kernel<DH, true>(),
+                                     dim3((unsigned)(rest * plan.splits)),
                                      dim3(one_shot_threads<DH>()), one_shot_smem<DH>(), st, tq, tk,
                                      tv, p) != cudaSuccess)
         return ECHO_ERR_CUDA;
@@ -1495,13 +1524,13 @@ echo_status launch_attention(const void *Q, int64_t ldq, const void *K, const vo
     if (M <= 0) return ECHO_OK;
     const int64_t items = ((int64_t)M + TILES * BM - 1) / (TILES * BM) * H;
     const int nb = (L + BN - 1) / BN;
-    const int splits = d == 64 ? choose_splits<64>(items, nb) : choose_splits<128>(items, nb);
-    if (L <= kItemsMaxKeys && splits == 1) {   // short key sets: the persistent kernel
+    const Plan plan = d == 64 ? choose_plan<64>(items, nb, L) : choose_plan<128>(items, nb, L);
+    if (L <= kItemsMaxKeys && plan.splits == 1) {   // short key sets: the persistent kernel
         if (d == 64) return launch_items_dh<64>(Q, ldq, K, V, ldkv, M, L, H, O, ldo, st);
         return launch_items_dh<128>(Q, ldq, K, V, ldkv, M, L, H, O, ldo, st);
     }
-    if (d == 64) return launch_dh<64>(Q, ldq, K, V, ldkv, M, L, H, splits, O, ldo, st);
-    return launch_dh<128>(Q, ldq, K, V, ldkv, M, L, H, splits, O, ldo, st);
+    if (d == 64) return launch_dh<64>(Q, ldq, K, V, ldkv, M, L, H, plan, O, ldo, st);
+    return launch_dh<128>(Q, ldq, K, V, ldkv, M, L, H, plan, O, ldo, st);
 }
 
 }  // namespace echo

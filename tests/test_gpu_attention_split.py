@@ -110,3 +110,16 @@ def test_attention_repeats(ec, M, L, H, d):
         bad += sum((o != ref).any().to(torch.int64) for o in outs)
     assert int(bad) == 0
     assert ec.echo_get_device_error() == 0
+
+
+@pytest.mark.parametrize("M,L,H,d", [
+    (256, 2049, 153, 64),    # a whole wave and one item over 8 CTAs, the last block of one key
+    (513, 2100, 52, 64),     # 156 items: four of the second launch, the last rows ragged
+    (257, 2200, 88, 128),    # 176 items: the first launch ends inside a head
+    (2560, 4000, 16, 64),    # 160 items: whole tiles
+    (700, 2049, 101, 64),    # 303 items: nearly two waves, one launch
+])
+def test_attention_last_wave(ec, M, L, H, d):
+    D = H * d
+    check(ec, G.random_rows(M, D, seed=M + d, scale=1.5),
+          G.random_rows(L, 2 * D, seed=L + d, scale=1.5), H, d)
