@@ -18,6 +18,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "extents.h"
 #include "internal.h"
 
 namespace {
@@ -298,7 +299,7 @@ __global__ void __launch_bounds__(kTopkThreads)
 topk_kernel(const float *__restrict__ scores, int NT, int K, int keys_in_smem,
             int32_t *__restrict__ idx) {
     pdl_enter();
-    extern __shared__ uint32_t skeys[];
+    extern __shared__ uint4 skeys4[];   // key_stage_bytes(NT)
     __shared__ int hist[3][2048];          // one per pass, cleared together
     __shared__ uint32_t sums[5][32];       // a block scan's or look-up's warp sums
     const int tid = threadIdx.x;
@@ -335,13 +336,13 @@ topk_kernel(const float *__restrict__ scores, int NT, int K, int keys_in_smem,
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int i = b + u * stride4;
-                if (i < NT) *reinterpret_cast<uint4 *>(skeys + i) = v[u];
+                if (i < NT) skeys4[i >> 2] = v[u];
             }
         }
     }
     __syncthreads();
     auto keys4 = [&](int i) -> uint4 {
-        return keys_in_smem ? *reinterpret_cast<const uint4 *>(skeys + i) : gkeys4(i);
+        return keys_in_smem ? skeys4[i >> 2] : gkeys4(i);
     };
 
     uint32_t prefix = 0, pmask = 0;
@@ -531,12 +532,12 @@ echo_status launch_topk(const float *keys, int NT, int K, int32_t *idx, cudaStre
         LaunchScope ls(ECHO_K_TOPK, NT, K, 0, st);
         if (launch_chained_cluster((unsigned)kTopkClusterCtas, topk_cluster_kernel,
                                    dim3(kTopkClusterCtas), dim3(kTopkThreads),
-                                   (size_t)slice * sizeof(uint32_t), st, keys, NT, K, slice,
+                                   key_stage_bytes(slice), st, keys, NT, K, slice,
                                    idx) != cudaSuccess)
             return ECHO_ERR_CUDA;
         return last_launch_status();
     }
-    const size_t key_bytes = (size_t)NT * sizeof(uint32_t);
+    const size_t key_bytes = key_stage_bytes(NT);
     const int in_smem = key_bytes <= (size_t)kTopkKeyBytesMax ? 1 : 0;
     LaunchScope ls(ECHO_K_TOPK, NT, K, 0, st);
     echo::launch_chained(topk_kernel, dim3(1), dim3(kTopkThreads), in_smem ? key_bytes : 0, st,
