@@ -248,7 +248,8 @@ size_t echo_cache_write_workspace_size(const echo_cache *c, int32_t n_rows);
 /* Writes src (bf16 [n_rows, D], device) into the cache at rows (int32
  * [n_rows], device, ascending and distinct), by the rules of c's form.
  * Errors: INVALID_ARG, SHAPE, WORKSPACE, CUDA; a non-finite row sets the
- * NONFINITE device flag (INT8, REF: as echo_cache_quant). */
+ * NONFINITE device flag (INT8, REF: as echo_cache_quant).  REF: seven rows are
+ * staged in a CTA's shared memory (227 KB); a D above 16592 returns SHAPE. */
 echo_status echo_cache_write(const echo_cache *c, const void *src, const int32_t *rows,
                              int32_t n_rows, void *workspace, size_t ws_bytes,
                              echo_stream_t stream);

@@ -19,6 +19,8 @@
 //                copies its row into its slot, a residual quantises x - r by the
 //                int8 rule, a run without a slot quantises x itself.
 // Reconstruction (read, merge) is one thread per 16 values: bf16(r + q s).
+#include <mutex>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -604,6 +606,33 @@ RefWs ref_ws(const echo_cache &c, void *ws, int32_t n) {
             reinterpret_cast<int32_t *>(p + 3 * a + b)};
 }
 
+size_t scan_smem_bytes(int D) { return (size_t)(kWin + 1) * D * sizeof(__nv_bfloat16); }
+
+// Dynamic shared memory that the scan may ask for on the current device (0: no
+// device): what a CTA may have beside its static buffers.  The kernel's limit is
+// raised to it once per device, whatever the width of the first write there, so that
+// no call depends on the widths written before it or by another thread meanwhile.
+size_t scan_smem_cap() {
+    static size_t cap[64] = {};
+    static std::mutex mu;
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    std::lock_guard<std::mutex> lk(mu);
+    if (!cap[dev]) {
+        cudaFuncAttributes fa;
+        int most = 0;
+        if (cudaFuncGetAttributes(&fa, ref_scan_kernel) != cudaSuccess ||
+            cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+            return 0;
+        const int dyn = most - (int)fa.sharedSizeBytes;
+        if (dyn <= 0 || cudaFuncSetAttribute(ref_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             dyn) != cudaSuccess)
+            return 0;
+        cap[dev] = (size_t)dyn;
+    }
+    return cap[dev];
+}
+
 }  // namespace
 
 namespace echo {
@@ -653,6 +682,11 @@ echo_status launch_cache_write(const echo_cache &c, const void *src, const int32
             s, rows, n, c.D, static_cast<__nv_bfloat16 *>(c.full), err);
         return last_launch_status();
     }
+    // before anything is enqueued: the release alone would leave slots counted free
+    // that the entries still name
+    const size_t scan_smem = scan_smem_bytes(c.D), scan_cap = scan_smem_cap();
+    if (!scan_cap) return ECHO_ERR_CUDA;
+    if (scan_smem > scan_cap) return ECHO_ERR_SHAPE;
     const RefWs w = ref_ws(c, ws, n);
     const int nseg = n_segments(c);
     if (cudaMemsetAsync(w.seg_lo, 0xFF, sizeof(int32_t) * (size_t)nseg, st) != cudaSuccess)
@@ -664,13 +698,8 @@ echo_status launch_cache_write(const echo_cache &c, const void *src, const int32
     }
     if (last_launch_status() != ECHO_OK) return ECHO_ERR_CUDA;
     {
-        const size_t smem = (size_t)(kWin + 1) * c.D * sizeof(__nv_bfloat16);
-        if (smem > 48 * 1024 &&
-            cudaFuncSetAttribute(ref_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem) != cudaSuccess)
-            return ECHO_ERR_CUDA;
         LaunchScope ls(ECHO_K_REF_SCAN, n, c.D, 0, st);
-        echo::launch_chained(ref_scan_kernel, dim3(nseg), dim3(kScanWarps * 32), smem, st, s,
+        echo::launch_chained(ref_scan_kernel, dim3(nseg), dim3(kScanWarps * 32), scan_smem, st, s,
                              w.seg_lo, w.seg_hi, c.tau, c.D,
                                                              w.src_pos);
     }

@@ -1,5 +1,9 @@
 """Cache writes and reads at the widths where a kernel holds more chunks of a row
 per thread, or falls back to reading it twice, bit for bit against the oracle."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -52,7 +56,7 @@ def test_quant_widths(ec, n, D):
         assert np.array_equal(got[keep], oracle.cache.dequant_gather(oq, os_)[keep])
 
 
-@pytest.mark.parametrize("D", [16, 1024, 1040, 2064, 5120, 5136, 8192, 8208])
+@pytest.mark.parametrize("D", [16, 1024, 1040, 2064, 3504, 5120, 5136, 8192, 8208, 16592])
 @pytest.mark.parametrize("R_cap", [40, 3])           # 3: runs without a slot, plain int8
 def test_ref_cache_widths(ec, D, R_cap):
     NT, seg = 60, 20
@@ -70,3 +74,37 @@ def test_ref_cache_widths(ec, D, R_cap):
         assert np.array_equal(g.t["scale"].cpu().numpy(), o.s)
         assert np.array_equal(g.t["ref"].cpu().numpy(), o.ref)
         assert np.array_equal(g.read().float().cpu().numpy(), o.reconstruct_bf16())
+
+
+FIRST_WRITE = """
+import sys, torch
+from paper_2608_02474_gb300 import echocache as ec
+c = ec.DeviceCache(ec.CACHE_REF, 24, 3504, seg_len=12)
+rows = torch.arange(24, dtype=torch.int32, device="cuda")
+for _ in range(2):
+    c.write(torch.randn(24, 3504, device="cuda").bfloat16(), rows)
+sys.exit(int(c.t["refcount"].sum()) != 24 or ec.echo_get_device_error())
+"""
+
+
+def test_ref_cache_first_write_of_a_process(ec):
+    """3504 is the width whose staged rows fit the 48 KB that need no raised limit only
+    without the scan's static buffers.  In a process of its own: a wider write before
+    it would have raised the limit."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.run([sys.executable, "-c", FIRST_WRITE], cwd=root, check=True, timeout=300)
+
+
+def test_ref_cache_too_wide_row_changes_nothing(ec):
+    """A row that the scan cannot stage is refused before anything is enqueued."""
+    D = 16608
+    c = ec.DeviceCache(ec.CACHE_REF, 8, D, seg_len=4)
+    c.load(ref=np.arange(8, dtype=np.int32), refcount=np.ones(8, np.int32))
+    before = {n: t.clone() for n, t in c.t.items() if n != "pool"}
+    with pytest.raises(ec.EchoError) as e:
+        c.write(torch.zeros(8, D, dtype=torch.bfloat16, device="cuda"),
+                torch.arange(8, dtype=torch.int32, device="cuda"))
+    assert e.value.status == 2                      # ECHO_ERR_SHAPE
+    torch.cuda.synchronize()
+    for n, t in before.items():
+        assert torch.equal(c.t[n], t), n
