@@ -26,6 +26,8 @@
 //               only when their row sum shows P above 2^64; final O / l to bf16.
 // Keys beyond L are masked to P = 0; queries beyond M run on zero rows and are
 // not stored.  Every mbarrier wait is bounded (ECHO_ERR_TIMEOUT).
+#include <cfloat>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -405,9 +407,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             };
             if (j == 0) {
                 m_used = block_max() * sl2;
-                // a CTA whose first keys all score -inf adds nothing to the sums
-                // of the others instead of NaN
-                if (SPLIT && m_used == -INFINITY) m_used = 0.f;
+                // a CTA whose first keys all score -inf: P = 0 there instead of NaN, and
+                // the first finite score of a later block overflows and brings its max
+                if (SPLIT && m_used == -INFINITY) m_used = -FLT_MAX;
             }
             float bsum = exp_pass();
             const bool redo = !(bsum <= 1.8446744e19f);     // > 2^64, inf or NaN
@@ -769,9 +771,9 @@ attn_d64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             };
             if (j == 0) {
                 m_used = row_max(half_max()) * sl2;
-                // a CTA whose first keys all score -inf adds nothing to the sums
-                // of the others instead of NaN
-                if (SPLIT && m_used == -INFINITY) m_used = 0.f;
+                // a CTA whose first keys all score -inf: P = 0 there instead of NaN, and
+                // the first finite score of a later block overflows and brings its max
+                if (SPLIT && m_used == -INFINITY) m_used = -FLT_MAX;
             }
             float bsum = exp_pass();
             const bool redo = !(bsum <= 1.8446744e19f);     // > 2^64, inf or NaN

@@ -91,6 +91,26 @@ def test_attention_split_maxima_differ(ec, d, lo, hi):
     check(ec, Q, np.concatenate([K, V], axis=1), H, d)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+def test_attention_split_first_keys_minus_infinity(ec, d):
+    """8 CTAs of four key blocks each; the first block of all but one scores -inf, and
+    every other score lies near -200 (in powers of two), far below 2^-126 of one: a
+    CTA has to take its maximum from the block after."""
+    H, M, L = 2, 150, 4000
+    D = H * d
+    g = np.random.default_rng(d)
+    Q = g.standard_normal((M, D)).astype(F32) * F32(0.3)
+    K = g.standard_normal((L, D)).astype(F32) * F32(0.3)
+    V = g.standard_normal((L, D)).astype(F32)
+    for h in range(H):
+        Q[:, h * d] = 1.0
+        K[:, h * d] = -200 / np.log2(np.e) * np.sqrt(d)
+        for r in range(1, 8):
+            K[512 * r:512 * r + 128, h * d] = -np.inf
+    Q, K, V = (G.to_bf16_values(a) for a in (Q, K, V))
+    check(ec, Q, np.concatenate([K, V], axis=1), H, d)
+
+
 @pytest.mark.parametrize("M,L,H,d", [(7800, 1000, 16, 64), (7800, 2100, 16, 64), (389, 2000, 16, 64),
                                      (3000, 2100, 8, 128)])
 def test_attention_repeats(ec, M, L, H, d):
