@@ -39,7 +39,8 @@ quant_kernel(const ST *__restrict__ src, const int32_t *__restrict__ rows, int n
     const int lane = threadIdx.x & 31;
     const int warps = blockDim.x >> 5;
     const int C = D >> 3;
-    for (int j = blockIdx.x * warps + (threadIdx.x >> 5); j < n_rows; j += gridDim.x * warps) {
+    for (RowWalk walk = grid_rows(warps); walk.below(n_rows); walk.next()) {
+        const int j = (int)walk.row;
         const ST *s = src + (int64_t)j * D;
         float amax = 0.f;
         bool nan = false, inf = false;
@@ -102,7 +103,8 @@ quant_regs_kernel(const __nv_bfloat16 *__restrict__ src, const int32_t *__restri
     const int lane = threadIdx.x & 31;
     const int warps = kQuantThreads / 32;
     const int C = D >> 3;
-    for (int j = blockIdx.x * warps + (threadIdx.x >> 5); j < n_rows; j += gridDim.x * warps) {
+    for (RowWalk walk = grid_rows(warps); walk.below(n_rows); walk.next()) {
+        const int j = (int)walk.row;
         const uint4 *s = reinterpret_cast<const uint4 *>(src + (int64_t)j * D);
         const int r = rows ? rows[j] : j;
         uint4 v[CPL];
@@ -134,7 +136,7 @@ quant_regs_kernel(const __nv_bfloat16 *__restrict__ src, const int32_t *__restri
 template <int CPL>
 void launch_quant_regs(const __nv_bfloat16 *src, const int32_t *rows, int n_rows, int D, int8_t *q,
                        float *scale, int *err, cudaStream_t st) {
-    const int grid = (n_rows + kQuantThreads / 32 - 1) / (kQuantThreads / 32);
+    const int grid = blocks_for_rows(n_rows, kQuantThreads / 32);
     echo::launch_chained(quant_regs_kernel<CPL>, dim3(grid), dim3(kQuantThreads), 0, st, src, rows,
                          n_rows, D, q, scale, err);
 }
@@ -167,8 +169,8 @@ __global__ void __launch_bounds__(kVecThreads)
 dequant_kernel(const int8_t *__restrict__ q, const float *__restrict__ scale,
                const int32_t *__restrict__ rows, int n_rows, int D, DT *__restrict__ dst) {
     pdl_enter();
-    for (PieceWalk w(D >> 4); w.row < n_rows; w.next()) {
-        const int r = rows ? rows[w.row] : w.row;
+    for (PieceWalk w = grid_pieces(D >> 4); w.below(n_rows); w.next()) {
+        const int r = rows ? rows[w.row] : (int)w.row;
         const int4 qv = __ldcs(reinterpret_cast<const int4 *>(q + (int64_t)r * D + 16 * w.piece));
         float f[16];
         dequant16(qv, scale[r], f);
@@ -202,12 +204,12 @@ dequant_merge_kernel(const int8_t *__restrict__ q, const float *__restrict__ sca
                      const int32_t *__restrict__ rowmap, const __nv_bfloat16 *__restrict__ y_act,
                      int NT, int D, __nv_bfloat16 *__restrict__ y) {
     pdl_enter();
-    PieceWalk w(D >> 4);
-    int pos_next = w.row < NT ? rowmap[w.row] : 0;   // a step ahead of the piece's own loads
-    while (w.row < NT) {
-        const int i = w.row, c = w.piece, pos = pos_next;
+    PieceWalk w = grid_pieces(D >> 4);
+    int pos_next = w.below(NT) ? rowmap[w.row] : 0;   // a step ahead of the piece's own loads
+    while (w.below(NT)) {
+        const int i = (int)w.row, c = (int)w.piece, pos = pos_next;
         w.next();
-        if (w.row < NT) pos_next = rowmap[w.row];
+        if (w.below(NT)) pos_next = rowmap[w.row];
         uint4 *o = reinterpret_cast<uint4 *>(y + (int64_t)i * D + 16 * c);
         if (pos >= 0) {
             if (y_act) {
@@ -238,12 +240,12 @@ merge_quant_kernel(int8_t *__restrict__ q, float *__restrict__ scale,
                    const int32_t *__restrict__ rowmap, const uint32_t *__restrict__ amax_bits,
                    int NT, int D, __nv_bfloat16 *__restrict__ y, int *err) {
     pdl_enter();
-    PieceWalk w(D >> 4);
-    int pos_next = w.row < NT ? rowmap[w.row] : 0;   // a step ahead of the piece's own loads
-    while (w.row < NT) {
-        const int i = w.row, c = w.piece, pos = pos_next;
+    PieceWalk w = grid_pieces(D >> 4);
+    int pos_next = w.below(NT) ? rowmap[w.row] : 0;   // a step ahead of the piece's own loads
+    while (w.below(NT)) {
+        const int i = (int)w.row, c = (int)w.piece, pos = pos_next;
         w.next();
-        if (w.row < NT) pos_next = rowmap[w.row];
+        if (w.below(NT)) pos_next = rowmap[w.row];
         uint4 *o = reinterpret_cast<uint4 *>(y + (int64_t)i * D + 16 * c);
         int4 *qr = reinterpret_cast<int4 *>(q + (int64_t)i * D + 16 * c);
         if (pos < 0) {

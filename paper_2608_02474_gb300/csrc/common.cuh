@@ -8,6 +8,7 @@
 #include <stdint.h>
 
 #include "../../include/echocache.h"
+#include "extents.h"
 
 #define ECHO_DEV __device__ __forceinline__
 
@@ -61,30 +62,15 @@ ECHO_DEV uint4 pack8_bf16(const float *f) {
     return u;
 }
 
-// A thread's walk over the pieces (row, piece of the row) of [n_rows, C] pieces in
-// steps of the whole grid, kept as row and piece: one division at the start instead
-// of a 64-bit division per piece, which was as long as moving the piece.
-struct PieceWalk {
-    int row, piece;
-    ECHO_DEV PieceWalk(int C) : C_(C) {
-        const unsigned t = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
-        row = (int)(t / (unsigned)C);
-        piece = (int)(t % (unsigned)C);
-        rows_ = (int)(step / (unsigned)C);
-        pieces_ = (int)(step % (unsigned)C);
-    }
-    ECHO_DEV void next() {
-        row += rows_;
-        piece += pieces_;
-        if (piece >= C_) {
-            piece -= C_;
-            ++row;
-        }
-    }
+// this thread's walk over pieces of rows of C pieces
+ECHO_DEV PieceWalk grid_pieces(int C) {
+    return PieceWalk(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, (unsigned)C);
+}
 
-  private:
-    int C_, rows_, pieces_;
-};
+// this warp's walk over rows, `warps` warps a block
+ECHO_DEV RowWalk grid_rows(int warps) {
+    return RowWalk{blockIdx.x * warps + (threadIdx.x >> 5), gridDim.x * warps};
+}
 
 ECHO_DEV uint64_t globaltimer_ns() {
     uint64_t t;

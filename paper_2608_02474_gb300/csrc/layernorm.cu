@@ -146,7 +146,8 @@ layernorm_warp_bf16(const __nv_bfloat16 *__restrict__ in, const int32_t *__restr
     const int warps = kThreads / 32;
     const int C = D >> 3;
     const float invD = 1.f / (float)D;
-    for (int j = blockIdx.x * warps + (threadIdx.x >> 5); j < n_rows; j += gridDim.x * warps) {
+    for (RowWalk walk = grid_rows(warps); walk.below(n_rows); walk.next()) {
+        const int j = (int)walk.row;
         const int r = rows ? rows[j] : j;
         const uint4 *src = reinterpret_cast<const uint4 *>(in + (int64_t)r * D);
         uint4 v[CPL];
@@ -340,8 +341,7 @@ template <int CPL>
 void launch_warp_bf16(const __nv_bfloat16 *in, const int32_t *rows, int n_rows, int D,
                       __nv_bfloat16 *out, __nv_bfloat16 *out2, const int32_t *idx, int n_idx,
                       int32_t *rowmap, uint32_t *zero, cudaStream_t st) {
-    constexpr int RPB = kThreads / 32;
-    int grid = (n_rows + RPB - 1) / RPB;
+    int grid = blocks_for_rows(n_rows, kThreads / 32);
     if (grid > 152 * 8) grid = 152 * 8;
     echo::launch_chained(layernorm_warp_bf16<CPL>, dim3(grid), dim3(kThreads), 0, st, in, rows,
                          n_rows, D, out, out2, idx, n_idx, rowmap, zero);
@@ -406,9 +406,8 @@ layernorm_warp_f32(const float *__restrict__ in, int n_rows, int D,
 
 template <int CPL>
 void launch_warp_f32(const float *in, int n_rows, int D, __nv_bfloat16 *out, cudaStream_t st) {
-    constexpr int RPB = kThreads / 32;
-    echo::launch_chained(layernorm_warp_f32<CPL>, dim3((n_rows + RPB - 1) / RPB), dim3(kThreads), 0,
-                         st, in, n_rows, D, out);
+    echo::launch_chained(layernorm_warp_f32<CPL>, dim3(blocks_for_rows(n_rows, kThreads / 32)),
+                         dim3(kThreads), 0, st, in, n_rows, D, out);
 }
 
 // fp32 rows of up to 8192 values: one CTA of 128 threads per row, the row in

@@ -509,8 +509,8 @@ __global__ void __launch_bounds__(kVec)
 cache_read_kernel(echo_cache c, const int32_t *__restrict__ rows, int n,
                   __nv_bfloat16 *__restrict__ dst) {
     pdl_enter();
-    for (PieceWalk w(c.D >> 4); w.row < n; w.next()) {
-        const int j = w.row, col = 16 * w.piece;
+    for (PieceWalk w = grid_pieces(c.D >> 4); w.below(n); w.next()) {
+        const int j = (int)w.row, col = 16 * (int)w.piece;
         const int i = rows ? rows[j] : j;
         uint4 o[2];
         reconstruct16<KIND>(c, i, col, o);
@@ -526,8 +526,8 @@ __global__ void __launch_bounds__(kVec)
 cache_merge_kernel(echo_cache c, const int32_t *__restrict__ rowmap,
                    const __nv_bfloat16 *__restrict__ y_act, __nv_bfloat16 *__restrict__ y) {
     pdl_enter();
-    for (PieceWalk w(c.D >> 4); w.row < c.NT; w.next()) {
-        const int i = w.row, col = 16 * w.piece;
+    for (PieceWalk w = grid_pieces(c.D >> 4); w.below(c.NT); w.next()) {
+        const int i = (int)w.row, col = 16 * (int)w.piece;
         const int pos = rowmap[i];
         uint4 *o = reinterpret_cast<uint4 *>(y + (int64_t)i * c.D + col);
         uint4 v[2];
@@ -549,8 +549,8 @@ cache_copy_kernel(const __nv_bfloat16 *__restrict__ src, const int32_t *__restri
                   int D, __nv_bfloat16 *__restrict__ full, int *err) {
     pdl_enter();
     bool bad = false;
-    for (PieceWalk w(D >> 3); w.row < n; w.next()) {
-        const int j = w.row, c = w.piece;
+    for (PieceWalk w = grid_pieces(D >> 3); w.below(n); w.next()) {
+        const int j = (int)w.row, c = (int)w.piece;
         const uint4 u = __ldcs(reinterpret_cast<const uint4 *>(src + (int64_t)j * D + 8 * c));
         bad |= bf16_nonfinite(u.x) || bf16_nonfinite(u.y) || bf16_nonfinite(u.z) ||
                bf16_nonfinite(u.w);

@@ -18,7 +18,6 @@
 #include <mutex>
 
 #include "common.cuh"
-#include "extents.h"
 #include "internal.h"
 
 namespace {
