@@ -30,3 +30,20 @@ def test_layernorm_widths(n, D, bf16):
     if bf16:
         assert torch.equal(ec.echo_layernorm(t, rows), ec.echo_layernorm(t))
     assert ec.echo_get_device_error() == 0
+
+
+@pytest.mark.parametrize("bf16", [True, False])
+@pytest.mark.parametrize("D", [256, 1024, 1032, 1536, 2048, 2056, 5120])
+def test_layernorm_of_a_row_whatever_comes_with_it(D, bf16):
+    """A row has the same bits alone, in a small batch and in a large one: from 1025 to
+    2048 fp32 values the kernel changes with the row count."""
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_2608_02474_gb300 import echocache as ec
+    g = torch.Generator(device="cuda").manual_seed(D)
+    x = torch.randn(3000, D, generator=g, device="cuda") * 2 + 0.5
+    x = x.bfloat16() if bf16 else x
+    out = ec.echo_layernorm(x)
+    for n in (1, 64, 1023, 1024, 1025):
+        assert torch.equal(ec.echo_layernorm(x[:n].contiguous()), out[:n])
+    assert ec.echo_get_device_error() == 0
