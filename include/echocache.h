@@ -497,7 +497,7 @@ echo_status echo_profile_enable(int32_t on);
  * the host arrays, clears the record list and returns the number copied (or
  * -1 on a CUDA error).  Shapes: GEMM (M, N, Kd; two projections in one
  * launch: (M1 + M2 N2 / N1, N1, Kd)); ATTENTION (M queries, L keys,
- * H * d); DRIFT (NT, D, 0); TOPK (NT, K, 0); LAYERNORM (rows, D, input element
+ * H * d; a call of two launches splits M between them by their work); DRIFT (NT, D, 0); TOPK (NT, K, 0); LAYERNORM (rows, D, input element
  * bytes); QUANT, DEQUANT, MERGE (rows, D, 0); ENERGY (T, frames, n_fft); STEP_DELTA (n, element bytes, 0)
  * for the reduction and (0, 0, blocks) for its final combine; UNIFORM (NT, K, 0);
  * REF_SCAN, REF_ALLOC, REF_STORE, CACHE_COPY (rows, D, 0); MERGE_QUANT (NT, D, K active

@@ -1501,18 +1501,22 @@ echo_status launch_dh(const void *Q, int64_t ldq, const void *K, const void *V, 
     p.err = echo::device_error_ptr();
     p.ntp = (M + TILES * BM - 1) / (TILES * BM);
     p.item0 = 0;
-    const int64_t rest = (int64_t)p.ntp * H - plan.whole;
-    echo::LaunchScope ls(ECHO_K_ATTENTION, M, L, (int64_t)H * DH, st);
-    if (plan.whole > 0)
+    const int64_t items = (int64_t)p.ntp * H, rest = items - plan.whole;
+    // recorded as queries over all heads: of two launches each by its share of the items
+    const int64_t m_whole = (int64_t)M * plan.whole / items;
+    if (plan.whole > 0) {
+        echo::LaunchScope ls(ECHO_K_ATTENTION, m_whole, L, (int64_t)H * DH, st);
         echo::launch_chained(one_shot_kernel<DH, false>(), dim3((unsigned)plan.whole),
                              dim3(one_shot_threads<DH>()), one_shot_smem<DH>(), st, tq, tk, tv, p);
+    }
     p.item0 = (int)plan.whole;
-    if (rest > 0 &&
+    if (rest > 0) {
+        echo::LaunchScope ls(ECHO_K_ATTENTION, M - m_whole, L, (int64_t)H * DH, st);
         echo::launch_chained_cluster((unsigned)plan.splits, one_shot_kernel<DH, true>(),
                                      dim3((unsigned)(rest * plan.splits)),
-                                     dim3(one_shot_threads<DH>()), one_shot_smem<DH>(), st, tq, tk,
-                                     tv, p) != cudaSuccess)
-        return ECHO_ERR_CUDA;
+                                     dim3(one_shot_threads<DH>()), one_shot_smem<DH>(), st, tq, tk, tv,
+                                     p);
+    }
     return echo::last_launch_status();
 }
 

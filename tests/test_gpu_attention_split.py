@@ -143,3 +143,23 @@ def test_attention_last_wave(ec, M, L, H, d):
     D = H * d
     check(ec, G.random_rows(M, D, seed=M + d, scale=1.5),
           G.random_rows(L, 2 * D, seed=L + d, scale=1.5), H, d)
+
+
+@pytest.mark.parametrize("M,L,H,d,launches", [
+    (513, 2100, 52, 64, 2), (257, 2200, 88, 128, 2), (7800, 7800, 16, 64, 2),
+    (700, 2049, 101, 64, 1), (389, 2000, 16, 64, 1), (300, 160, 16, 64, 1),
+])
+def test_attention_launches_are_counted(ec, M, L, H, d, launches):
+    """Every kernel of a call is counted and recorded; the records' queries add up."""
+    import torch
+    D = H * d
+    Q = torch.zeros(M, D, dtype=torch.bfloat16, device="cuda")
+    KV = torch.zeros(L, 2 * D, dtype=torch.bfloat16, device="cuda")
+    ec.echo_profile_read()
+    n0 = ec.echo_launch_count()
+    ec.echo_profile_enable(True)
+    ec.echo_attention(Q, KV[:, :D], KV[:, D:], H, d)
+    ec.echo_profile_enable(False)
+    rec = ec.echo_profile_read()
+    assert ec.echo_launch_count() - n0 == launches == len(rec)
+    assert sum(r[1] for r in rec) == M and all(r[1] > 0 and r[2:4] == (L, D) for r in rec)
