@@ -139,8 +139,14 @@ def _p(t):
 
 
 # The current stream's handle without the Stream object around it, which costs as
-# much host time as a kernel launch (3.1 us of an 18 us call; this takes 0.3).
-_raw_stream, _cur_device = torch._C._cuda_getCurrentRawStream, torch.cuda.current_device
+# much host time as a kernel launch (3.1 us of an 18 us call; this takes 0.3).  Where
+# PyTorch does not have the name (a build without CUDA, another version), by the object.
+def _stream_handle(device):
+    return torch.cuda.current_stream(device).cuda_stream
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", _stream_handle)
+_cur_device = torch.cuda.current_device
 
 
 def _stream(stream=None):

@@ -5,10 +5,12 @@ CPU fallback.  No GPU.
   the oracle imports nothing of the package.
 - The seeded input generators (synth/) import neither.
 - The binding fails loudly, before any compute, when the library is missing.
+- It can be imported with a PyTorch that has no raw handle of the current stream.
 """
 import ast
 import glob
 import os
+import sys
 
 import pytest
 
@@ -58,3 +60,24 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(ec, "LIB_PATH", str(tmp_path / "missing.so"))
     with pytest.raises(RuntimeError, match="missing"):
         ec.lib()
+
+
+def test_import_without_the_raw_stream_name(monkeypatch):
+    """A PyTorch built without CUDA lacks it: the import still works, and the handle comes
+    from the Stream object."""
+    import importlib.util
+
+    import torch
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    spec = importlib.util.spec_from_file_location(
+        "echocache_without_raw_stream", os.path.join(ROOT, PKG, "echocache.py"))
+    ec = importlib.util.module_from_spec(spec)
+    monkeypatch.setitem(sys.modules, spec.name, ec)
+    spec.loader.exec_module(ec)
+
+    class Stream:
+        cuda_stream = 77
+
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda device=None: Stream)
+    monkeypatch.setattr(ec, "_cur_device", lambda: 0)
+    assert ec._stream() == 77 and ec._stream(Stream) == 77
