@@ -36,7 +36,7 @@ namespace {
 constexpr int BM = 128;        // queries per tile; two tiles per CTA
 constexpr int TILES = 2;
 constexpr int BN = 128;        // keys per block
-constexpr int RING_MAX = 8;    // K/V ring slots (K_j and V_j alternate)
+constexpr int RING_MAX = 8;    // most K/V ring slots of the persistent kernel
 constexpr int PAIRS = 3;       // barriers of the pairs (V_j, K_{j+1}) in the ring
 constexpr int THREADS = 384;   // 4 control warps + 2 softmax warpgroups
 constexpr uint32_t TMEM_COLS = 512;   // S0, S1, O0, O1
@@ -53,11 +53,12 @@ struct Cfg {
     static constexpr int ATOMS = DH / 64;
     static constexpr int Q_BYTES = BM * DH * 2;
     static constexpr int SLOT_BYTES = BN * DH * 2;
-    static constexpr int RING = DH == 128 ? 5 : RING_MAX;
-    static constexpr int SMEM = TILES * Q_BYTES + RING * SLOT_BYTES + 1024;
     static constexpr uint32_t IDESC_S = idesc_bf16_f32(BM, BN);
     static constexpr uint32_t IDESC_PV = idesc_bf16_f32(BM, DH) | (1u << 16);  // B MN-major
 };
+
+constexpr int D128_RING = 5;   // K/V slots of attn_tc_kernel
+constexpr int D128_SMEM = TILES * Cfg<128>::Q_BYTES + D128_RING * Cfg<128>::SLOT_BYTES + 1024;
 
 struct AttnParams {
     int M, L;
@@ -103,11 +104,11 @@ ECHO_DEV void sum_split_rows(const AttnParams &p, uint32_t stage_addr, int split
     }
 }
 
-template <int DH, int HALVES>
+template <int DH, int HALVES, int RING_BYTES>
 ECHO_DEV void combine_splits(const AttnParams &p, uint8_t *stage, float2 *own_ml, int half,
                              uint32_t o_tmem, int row, float m_own, float l_own, bool ok, int splits, int split,
                              int q0, int h) {
-    static_assert(TILES * BM * DH * 4 <= Cfg<DH>::RING * Cfg<DH>::SLOT_BYTES, "staged over the ring");
+    static_assert(TILES * BM * DH * 4 <= RING_BYTES, "staged over the ring");
     if (l_own == 0.f) m_own = -INFINITY;
     if (half == 0) *own_ml = make_float2(m_own, l_own);
     __syncwarp();
@@ -146,21 +147,22 @@ ECHO_DEV void combine_splits(const AttnParams &p, uint8_t *stage, float2 *own_ml
     cluster_sync_all();   // no CTA leaves while another may still read its rows
 }
 
-template <int DH, bool SPLIT>
+template <bool SPLIT>
 __global__ void __launch_bounds__(THREADS, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
-    using C = Cfg<DH>;
+    using C = Cfg<128>;
+    constexpr int DH = 128;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                 ~static_cast<uintptr_t>(1023));
-    constexpr int RING = C::RING;
+    constexpr int RING = D128_RING;
     uint8_t *Qs = smem;                                  // [TILES][Q_BYTES]
     uint8_t *Ring = Qs + TILES * C::Q_BYTES;             // [RING][SLOT_BYTES]
 
     // Every barrier is reused only after its previous phase has been observed
     // by its waiter, so no waiter can fall two phases behind.
-    __shared__ __align__(8) uint64_t q_full, pair_full[PAIRS], ring_empty[RING_MAX];
+    __shared__ __align__(8) uint64_t q_full, pair_full[PAIRS], ring_empty[RING];
     __shared__ __align__(8) uint64_t s_full[TILES], p_full[TILES], pv_done[TILES];
     __shared__ __align__(8) uint64_t drain;
     __shared__ uint32_t tmem_slot;
@@ -449,10 +451,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         if (ok) tc_fence_after();
         if constexpr (SPLIT) {
             // the rows' maxima and sums in the tile's Q, the scaled rows over the ring
-            combine_splits<DH, 1>(p, Ring,
-                                  reinterpret_cast<float2 *>(Qs + t * C::Q_BYTES) + quad * 32 + lane, 0,
-                                  tmem + lane_base + o_col, t * BM + quad * 32 + lane, m_used, l, ok,
-                                  splits, split, q0, h);
+            combine_splits<DH, 1, RING * C::SLOT_BYTES>(
+                p, Ring, reinterpret_cast<float2 *>(Qs + t * C::Q_BYTES) + quad * 32 + lane, 0,
+                tmem + lane_base + o_col, t * BM + quad * 32 + lane, m_used, l, ok, splits, split, q0, h);
         } else if (ok) {
             const float inv = 1.f / l;
             // The warp's 32 rows of O go through its quarter of Q_t (free now:
@@ -536,7 +537,7 @@ attn_d64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 
     // Every barrier is reused only after its previous phase has been observed
     // by its waiter, so no waiter can fall two phases behind.
-    __shared__ __align__(8) uint64_t q_full, ring_full[RING_MAX], ring_empty[RING_MAX];
+    __shared__ __align__(8) uint64_t q_full, ring_full[RING], ring_empty[RING];
     __shared__ __align__(8) uint64_t s_full[S_BUFS], p_full[S_BUFS], pv_done[TILES], o_done[TILES];
     __shared__ __align__(8) uint64_t drain;
     __shared__ uint32_t tmem_slot;
@@ -838,9 +839,9 @@ attn_d64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         l = row_x[t][0][row] + row_x[t][1][row];
         if constexpr (SPLIT) {
             // the rows' maxima and sums in the tile's Q, the scaled rows over the ring
-            combine_splits<DH, 2>(p, Ring, reinterpret_cast<float2 *>(Qs + t * C::Q_BYTES) + row, half,
-                               tmem + lane_base + o_col, t * BM + row, m_used, l, ok, splits, split,
-                               q0, h);
+            combine_splits<DH, 2, RING * PAIR_BYTES>(
+                p, Ring, reinterpret_cast<float2 *>(Qs + t * C::Q_BYTES) + row, half,
+                tmem + lane_base + o_col, t * BM + row, m_used, l, ok, splits, split, q0, h);
         } else if (ok) {
             const float inv = 1.f / l;
             // The 32 rows of O go through their quarter of Q_t (free now: every
@@ -1380,12 +1381,12 @@ constexpr int kTailFixed = 4;  // a second launch, in the key-block times of cho
 template <int DH, bool SPLIT>
 constexpr auto one_shot_kernel() {
     if constexpr (DH == 64) return attn_d64_kernel<SPLIT>;
-    else return attn_tc_kernel<DH, SPLIT>;
+    else return attn_tc_kernel<SPLIT>;
 }
 template <int DH>
 constexpr int one_shot_threads() { return DH == 64 ? D64_THREADS : THREADS; }
 template <int DH>
-constexpr int one_shot_smem() { return DH == 64 ? D64_SMEM : Cfg<DH>::SMEM; }
+constexpr int one_shot_smem() { return DH == 64 ? D64_SMEM : D128_SMEM; }
 
 // it may take its dynamic shared memory (once per device)
 template <int DH>

@@ -436,20 +436,6 @@ ECHO_DEV void tmem_st16(uint32_t taddr, const uint32_t *r) {
 
 ECHO_DEV void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Shared-memory descriptor for an MN-major bf16 operand written by TMA with
-// 128-byte swizzle: 64 MN-contiguous elements per 128-byte row, K rows 128 B
-// apart, 8-row K groups `sbo` bytes apart, MN atoms of 64 elements `lbo` apart.
-ECHO_DEV uint64_t smem_desc_sw128_mn(const void *p, uint32_t lbo, uint32_t sbo) {
-    const uint64_t addr = smem_u32(p);
-    uint64_t d = 0;
-    d |= (addr & 0x3FFFFull) >> 4;
-    d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
-
 // packed fp32 pairs (sm_100 family): one instruction for two lanes of work
 ECHO_DEV uint64_t f2_pack(float a, float b) {
     uint64_t r;
@@ -479,19 +465,6 @@ ECHO_DEV float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
-}
-
-// Shared-memory matrix descriptor for a K-major bf16 tile written by TMA with
-// 128-byte swizzle: rows of 64 elements (128 B), 8-row groups 1024 B apart.
-ECHO_DEV uint64_t smem_desc_sw128(const void *p) {
-    const uint64_t addr = smem_u32(p);
-    uint64_t d = 0;
-    d |= (addr & 0x3FFFFull) >> 4;           // start address, 16-byte units
-    d |= (uint64_t)(16 >> 4) << 16;          // leading byte offset (unused for SW128 K-major)
-    d |= (uint64_t)(1024 >> 4) << 32;        // stride byte offset: 8 rows x 128 B
-    d |= (uint64_t)1 << 46;                  // descriptor version (sm_100 family)
-    d |= (uint64_t)2 << 61;                  // layout: 128-byte swizzle
-    return d;
 }
 
 // Instruction descriptor, kind::f16: bf16 A and B (K-major), fp32 D, M x N.
