@@ -301,8 +301,13 @@ ECHO_DEV float4 ld_shared_cluster_f4(uint32_t cluster_addr) {
 
 // Arrive on an mbarrier given by its shared::cluster address (possibly another
 // CTA's) without a release: it orders no earlier memory access, so the thread does
-// not wait for its global stores.  For handing back tensor memory whose loads have
-// completed (tcgen05.wait::ld, then tcgen05.fence::before_thread_sync).
+// not wait for its global stores.  Only for handing back tensor memory, and that
+// rests on three things done before it, not on the arrival: the loads have put
+// their values into registers (tcgen05.wait::ld), tcgen05.fence::before_thread_sync
+// orders them before what this thread does next, and the thread that issues the MMAs
+// passes tcgen05.fence::after_thread_sync once it has seen the phase.  The arriving
+// lane speaks for its warp: the loads and the wait are warp-wide (.sync.aligned),
+// and a __syncwarp lies between.
 ECHO_DEV void mbar_arrive_remote_relaxed(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr)
                  : "memory");

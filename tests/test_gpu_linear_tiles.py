@@ -64,3 +64,42 @@ def test_linear_epilogues(ec, M, Kd, N):
     close(host(wide[:, :N]), lin - b, **h_tol)
     assert bool((wide[:, N:] == 7).all())
     assert ec.echo_get_device_error() == 0
+
+
+def test_gelu_of_every_bf16_value(ec):
+    """GELU over every bf16 value, both output forms (bf16: one exponential and one
+    quotient; fp32: tanhf).  The projection passes each value through unchanged.
+
+    bf16: x / (1 + 2^w), w = -2 u log2(e), |w| <= 126 where the result is not below the
+    smallest normal number.  Four fp32 roundings make w (2^-24 each, of which the ones of
+    x^2 and of its factor count at most once), so 2^w is off by at most
+    126 ln 2 * 4 * 2^-24 = 2.1e-5 of itself, the exponential and the quotient by 2 ulp;
+    then the rounding to bf16's 8 bits, at most 2^-8.  Results below 11 * 2^-126 may vanish."""
+    bits = torch.arange(65536, dtype=torch.int32).to(torch.uint16)
+    x = bits.view(torch.bfloat16)
+    A = torch.zeros(65536, 64, dtype=torch.bfloat16)
+    A[:, 0] = x
+    W = torch.zeros(64, 64, dtype=torch.bfloat16)
+    W[:, 0] = 1
+    A, W = A.cuda(), W.cuda()
+    got16 = ec.echo_linear(A, W, None, act=1)
+    got32 = ec.echo_linear(A, W, None, act=1, out_dtype=torch.float32)
+    assert bool((got16.view(torch.uint16) == got16.view(torch.uint16)[:, :1]).all())
+    # what the two forms make of infinities and NaN: the same
+    assert torch.equal(torch.isnan(got16), torch.isnan(got32))
+    assert torch.equal(torch.isinf(got16), torch.isinf(got32))
+    g = got16[:, 0].double().cpu()
+    v = x.double()
+    fin = torch.isfinite(v)
+    assert torch.isnan(g[torch.isnan(v)]).all()
+    assert g[v == float("inf")] == float("inf") and torch.isnan(g[v == float("-inf")])
+    assert torch.isfinite(g[fin]).all()
+    v, g = v[fin], g[fin]
+    u = np.sqrt(2 / np.pi) * (v + 0.044715 * v ** 3)
+    exact = v / (1 + torch.exp(-2 * u))             # (1 + tanh u) / 2 without its cancellation
+    assert bool(((g - exact).abs() <= (2 ** -8 + 3e-5) * exact.abs() + 11 * 2.0 ** -126).all())
+    # and as often the bf16 value next to the exact one as the tanhf form rounded to bf16
+    nearest = exact.float().bfloat16().double()
+    old = got32[:, 0].bfloat16().double().cpu()[fin]
+    assert int((g != nearest).sum()) <= int((old != nearest).sum())
+    assert ec.echo_get_device_error() == 0
