@@ -377,15 +377,20 @@ ATTN_CASES = [
     (128, 64, 4, 128),
     (130, 672, 3, 128),
     (64, 7800, 2, 64),
-    # key sets up to 2048 take the persistent kernel (items chained per SM)
+    # key sets up to 2048 take the persistent kernel (items chained per SM), unless few
+    # (tile pair, head) items leave SMs idle and their keys are split over a cluster
     (6552, 672, 40, 128),    # cross-attention of the 32760-token block: 1040 items, 96-key blocks
     (3000, 160, 16, 64),     # 192 items (some CTAs take two), 96-key blocks with a masked tail
     (1000, 64, 4, 128),      # 64-key blocks
     (300, 32, 3, 64),        # 32-key blocks
-    (300, 2048, 2, 128),     # the largest key set of the persistent kernel
-    (300, 2049, 2, 128),     # one key more: the one-shot kernel
+    (300, 2048, 2, 128),     # four items: keys over 8 CTAs
+    (300, 2049, 2, 128),     # one key more: a block of one key
     (300, 4096, 2, 64),
     (300, 4097, 2, 64),
+    (600, 2048, 40, 128),    # the largest key set of the persistent kernel, 120 items
+    (600, 2048, 40, 64),
+    (600, 2000, 40, 64),     # the same with a masked last block
+    (800, 2049, 40, 128),    # one key more, 160 items: the one-shot kernel
 ]
 
 
@@ -406,8 +411,19 @@ def test_attention(ec, M, L, H, d):
 def test_attention_running_max_jumps(ec, d):
     """Later key blocks whose logits exceed the first block's by far more than
     2^64 force the kernel's rescale path (running max refreshed, O and the row
-    sum rescaled in tensor memory); the result must still match the oracle."""
-    H, M, L = 2, 150, 700
+    sum rescaled in tensor memory); the result must still match the oracle.
+    Two items: the keys are split over a cluster."""
+    running_max_jumps(ec, 2, 150, 700, d)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_attention_running_max_jumps_persistent(ec, d):
+    """The same in the persistent kernel: 200 items on 152 SMs, so that a CTA's second
+    item rescales while its first item's rows are still being stored."""
+    running_max_jumps(ec, 40, 1100, 700, d)
+
+
+def running_max_jumps(ec, H, M, L, d):
     D = H * d
     g = np.random.default_rng(d)
     Q = np.full((M, D), 2.0, dtype=F32) + g.standard_normal((M, D)).astype(F32) * F32(0.05)
