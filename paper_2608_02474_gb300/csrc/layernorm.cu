@@ -18,7 +18,7 @@ constexpr int kMaxChunks = 8;
 // Up to this width a warp holds a row in its registers and every row gets a warp of
 // its own: short rows are bound by latency, and streaming them two at a time per
 // warp, or one per CTA, kept too few loads in flight.  7800 rows of 1024: bf16 13.0
-// -> 4.4 us, fp32 16.7 -> 5.0 us; 63960 rows of 2048: 97 -> 80, 154 -> 112 us.  At
+// -> 4.4 us, fp32 16.7 -> 4.9 us; 63960 rows of 2048: 97 -> 80, 154 -> 112 us.  At
 // 3072 the streaming forms are as fast (7800 rows: 15.5 us against 17.8).
 constexpr int kWarpRowMax = 2048;
 
@@ -367,39 +367,42 @@ void launch_regs_bf16(const __nv_bfloat16 *in, const int32_t *rows, int n_rows, 
 // steps each quarter of the warp works on one of them: 18 shuffles a row instead of
 // 40 (7800 rows of 2048 13.2 -> 11.6 us; 10.5 with one sum per lane in an order of
 // its own).
-template <int P>
-ECHO_DEV float ordered_total(const float *p) {
+ECHO_DEV float ordered_total(const float (&p)[4]) {
     const int lane = threadIdx.x & 31;
     auto xor_add = [](float keep, float pass, int o) { return keep + __shfl_xor_sync(0xffffffffu, pass, o); };
     const bool hi = lane & 16, odd = lane & 8;
-    float t;
-    if (P == 4) {
-        const float a = xor_add(hi ? p[P - 2] : p[0], hi ? p[0] : p[P - 2], 16);
-        const float b = xor_add(hi ? p[P - 1] : p[1], hi ? p[1] : p[P - 1], 16);
-        t = xor_add(odd ? b : a, odd ? a : b, 8);
-    } else {
-        t = xor_add(hi ? p[1] : p[0], hi ? p[0] : p[1], 16);
-        t = xor_add(t, t, 8);
-    }
+    const float a = xor_add(hi ? p[2] : p[0], hi ? p[0] : p[2], 16);
+    const float b = xor_add(hi ? p[3] : p[1], hi ? p[1] : p[3], 16);
+    float t = xor_add(odd ? b : a, odd ? a : b, 8);
     t = xor_add(t, t, 4);
     t = xor_add(t, t, 2);
     t = xor_add(t, t, 1);
     float r = __shfl_sync(0xffffffffu, t, 0);
 #pragma unroll
-    for (int w = 1; w < P; ++w) r += __shfl_sync(0xffffffffu, t, w * (32 / P));
+    for (int w = 1; w < 4; ++w) r += __shfl_sync(0xffffffffu, t, 8 * w);
     return r;
 }
 
+// the sum of p[0] over the warp as a xor butterfly adds it
+ECHO_DEV float ordered_total(const float (&p)[1]) {
+    float s = p[0];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
 // fp32 rows of up to kWarpRowMax values: one warp per row, the row in registers
-// (lane l holds 16-byte chunks l, l + 32, ...).  Sums in the order of
-// layernorm_row_f32 below, to the same bits, so that a row's result does not depend on
-// how many rows come with it: chunk l + 32 k belongs to thread l of warp k mod 4 there,
-// and a lane keeps the partial sums of the four.
+// (lane l holds 16-byte chunks l, l + 32, ...).  Sums: up to 1024 values each lane's
+// chunks in order, then a xor butterfly.  Above, where a few rows take
+// layernorm_row_f32 below, in the order of that form, to the same bits, so that a
+// row's result does not depend on how many rows come with it: chunk l + 32 k belongs
+// to thread l of warp k mod 4 there, and a lane keeps the partial sums of the four.
 template <int CPL>
 __global__ void __launch_bounds__(kThreads)
 layernorm_warp_f32(const float *__restrict__ in, int n_rows, int D,
                    __nv_bfloat16 *__restrict__ out) {
     pdl_enter();
+    constexpr int P = CPL > 8 ? 4 : 1;
     const int lane = threadIdx.x & 31;
     const int j = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
     if (j >= n_rows) return;
@@ -410,24 +413,30 @@ layernorm_warp_f32(const float *__restrict__ in, int n_rows, int D,
 #pragma unroll
     for (int k = 0; k < CPL; ++k)
         v[k] = lane + 32 * k < C4 ? __ldcs(row + lane + 32 * k) : make_float4(0.f, 0.f, 0.f, 0.f);
-    constexpr int P = CPL < 4 ? CPL : 4;   // warps of that form with chunks
-    static_assert(P == 2 || P == 4, "total");
     float s[P] = {};
 #pragma unroll
     for (int k = 0; k < CPL; ++k) {
         float &p = s[k % P];
-        p += v[k].x; p += v[k].y; p += v[k].z; p += v[k].w;
+        if constexpr (P == 1) {
+            p += (v[k].x + v[k].y) + (v[k].z + v[k].w);
+        } else {
+            p += v[k].x; p += v[k].y; p += v[k].z; p += v[k].w;
+        }
     }
-    const float mean = ordered_total<P>(s) * invD;
+    const float mean = ordered_total(s) * invD;
     float ss[P] = {};
 #pragma unroll
     for (int k = 0; k < CPL; ++k)
         if (lane + 32 * k < C4) {
             const float a = v[k].x - mean, b = v[k].y - mean, c = v[k].z - mean, d = v[k].w - mean;
             float &p = ss[k % P];
-            p += a * a; p += b * b; p += c * c; p += d * d;
+            if constexpr (P == 1) {
+                p += (a * a + b * b) + (c * c + d * d);
+            } else {
+                p += a * a; p += b * b; p += c * c; p += d * d;
+            }
         }
-    const float rstd = rsqrtf(ordered_total<P>(ss) * invD + 1e-6f);
+    const float rstd = rsqrtf(ordered_total(ss) * invD + 1e-6f);
     uint2 *dst = reinterpret_cast<uint2 *>(out + (int64_t)j * D);
 #pragma unroll
     for (int k = 0; k < CPL; ++k)
