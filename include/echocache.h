@@ -453,6 +453,8 @@ echo_status echo_linear(const void *A, int64_t lda, int32_t M, int32_t Kd,
 /* O[m, h d + e] = sum_j softmax_j(Q_h[m] . K_h[j] / sqrt(d)) V_h[j, e]:
  *   Q bf16 [M, ldq], K and V bf16 [L, ldkv] (head h at columns h d .. h d + d - 1),
  *   O bf16 [M, ldo].  d in {64, 128}; strides multiples of 8.
+ * The same call gives the same bits every time; how its keys are divided between
+ * CTAs, and with it the order of the sums, depends on M, L, H and d.
  * Errors: INVALID_ARG, SHAPE, CUDA. */
 echo_status echo_attention(const void *Q, int64_t ldq, const void *K, const void *V,
                            int64_t ldkv, int32_t M, int32_t L, int32_t H, int32_t d,
