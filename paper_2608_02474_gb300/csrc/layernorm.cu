@@ -217,6 +217,7 @@ layernorm_warp_bf16(const __nv_bfloat16 *__restrict__ in, const int32_t *__restr
 // >= 0: the LN of every latent (for K and V) then also yields the gathered LN
 // of the active ones (for Q') without reading them a second time.
 constexpr int kBulkWarps = 4;
+constexpr size_t kBulkSmemMin = 78 * 1024;   // a third of an SM's 228 KB and more: two CTAs per SM
 
 template <int CPL>
 __global__ void __launch_bounds__(kBulkWarps * 32)
@@ -321,7 +322,11 @@ layernorm_bulk_bf16(const __nv_bfloat16 *__restrict__ in, int n_rows, int D,
 template <int CPL>
 void launch_bulk_bf16(const __nv_bfloat16 *in, int n_rows, int D, __nv_bfloat16 *out,
                       const int32_t *scatter_map, __nv_bfloat16 *out2, cudaStream_t st) {
-    const size_t smem = (size_t)kBulkWarps * 2 * D * sizeof(__nv_bfloat16);
+    // Two CTAs per SM, as the grid has them, whatever the width: where four would fit,
+    // the next kernel's CTAs came to lie unevenly beside those still running (32760 rows
+    // of 2112 59.0 -> 51.5 us, 7800 of 3072 19.0 -> 17.9, 15000 of 4096 44.3 -> 42.8).
+    size_t smem = (size_t)kBulkWarps * 2 * D * sizeof(__nv_bfloat16);
+    if (smem < kBulkSmemMin) smem = kBulkSmemMin;
     static int attr_done[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
