@@ -479,19 +479,23 @@ echo_status run_bn(const Problem &x, const Problem &y, cudaStream_t st) {
     return echo::last_launch_status();
 }
 
-// Tile width, by the cycles of the waves: a 64-deep k-block of 256 columns takes
-// 512 (the tensor rate), of 128 columns about 340 (the copies into shared memory),
-// plus about 600 a tile and the last tile's epilogue, which nothing overlaps.  128
-// columns spread a small output over more SM pairs: 1560 x 1024 x 1024 12.8 ->
-// 10.3 us, 1560 x 1024 x 4096 25.7 -> 21.4 us, 400 x 640 x 2048 16.8 -> 13.4 us,
-// 1563 x 4096 x 1024 25.5 -> 23.2 us; at 7800 x 1024 x 4096 they take 69 us
-// against 48, at 600 x 5120 x 5120 44 against 31, and the rule keeps 256.
+// Tile width, by the cycles of the waves with every SM pair at work: a 64-deep k-block
+// of 256 columns takes 512 (0.262 us), of 128 columns 440 (0.225 us: the copies into
+// shared memory, which the pairs share the L2 for), plus a tile's own part and the
+// last tile's epilogue, which nothing overlaps.  So 128 columns gain where they spread
+// a small output over pairs that would be idle, or save most of a wave.  Of 3901
+// measured calls (M 16 .. 20000, N 128 .. 13824, depth 128 .. 5120; plain, GELU, fp32
+// residual) the choice is 0.1% from the better width on average; by more than 8% it
+// is 12 times (16 rows at depth 3072; GELU or a residual at depth 512, 3 waves for 2).
+// 256 against 128 columns: 1560 x 1024 x 1024 9.8 and 8.6 us, 1560 x 1024 x 4096 22.5
+// and 19.7, 400 x 640 x 2048 13.8 and 11.3; 1560 x 4096 x 1024 14.9 and 17.3, 2560 x
+// 2048 x 5120 48.6 and 60.3, 600 x 5120 x 5120 28.1 and 41.8.
 bool narrow_tiles(int M, int N, int Kd, int M2 = 0, int N2 = 0) {
     const int64_t pairs = num_sms() / 2, kb = Kd / BK;
     const int64_t nm = (M + 2 * BM - 1) / (2 * BM), nm2 = (M2 + 2 * BM - 1) / (2 * BM);
     const int64_t w256 = (nm * ((N + 255) / 256) + nm2 * ((N2 + 255) / 256) + pairs - 1) / pairs;
     const int64_t w128 = (nm * ((N + 127) / 128) + nm2 * ((N2 + 127) / 128) + pairs - 1) / pairs;
-    return w128 * (kb * 340 + 600) + 1500 < w256 * (kb * 512 + 600) + 3000;
+    return w128 * (kb * 440 + 900) < w256 * (kb * 512 + 1800) + 500;
 }
 
 bool make_problem(const echo::LinearArgs &a, bool narrow, Problem &x) {
