@@ -7,8 +7,8 @@
 //                decrement of the slot's count) and the bounds of each scan
 //                segment's written rows are recorded;
 //   ref_scan     one CTA per scan segment walks its written rows in token
-//                order, 6 rows a round: the rows are staged in shared memory,
-//                the 12 warps compute the fp32 cosines the walk is likely to need
+//                order, 6 or 12 rows a round: the rows are staged in shared memory,
+//                two warps per row compute the fp32 cosines the walk is likely to need
 //                (each row against the entering reference and against the row
 //                before it, canonical order), then one thread walks the rows,
 //                asking for others where it must, and the last new reference
@@ -26,8 +26,11 @@
 
 namespace {
 
-constexpr int kWin = 6;             // rows of a scan window
-constexpr int kScanWarps = 2 * kWin;
+// Rows of a scan window: 6, or 12 where every segment has an SM to itself and the time
+// is one segment's walk.  A write of 7800 rows in 150 segments of 52, six rows against
+// twelve: 43 and 39 us at 128 values, 117 and 89 at 5120 (nearly every row a reference:
+// 49 and 45, 125 and 97); 9000 rows in 174 segments: 47 and 58, 126 and 131.
+constexpr int kWin = 6, kWinWide = 12, kWideSegments = 152;
 constexpr int kAllocThreads = 1024;
 constexpr int kStoreThreads = 256;
 constexpr int kVec = 256;
@@ -98,29 +101,30 @@ ECHO_DEV void warp_dot(const uint4 *a, const uint4 *b, int C, int lane, bool nor
 
 // src_pos[j] = position (in rows) of row j's reference; j itself for a reference.
 //
-// One CTA per scan segment.  The segment's written rows are taken kWin at a
+// One CTA per scan segment.  The segment's written rows are taken WIN at a
 // time: the window's rows are staged in shared memory, then every row is compared
 // with the reference that the window was entered with and with the row before it,
 // one similarity per warp, and one thread walks the window in order.  Those two
 // suffice while the reference stays or changes at every row; a row that follows a
 // change by two or more also needs its similarity to the row of the change, which
 // is then computed for the rest of the window at once before the walk goes on.
-// Dynamic shared memory: kWin window rows, then the current reference row (bf16, D
+// Dynamic shared memory: WIN window rows, then the current reference row (bf16, D
 // each); six rows leave room for three CTAs per SM at D = 5120.  6552 rows of 5120:
 // 70 us with all 36 similarities of windows of eight rows and two CTAs per SM, 49 us.
-__global__ void __launch_bounds__(kScanWarps * 32)
+template <int WIN>
+__global__ void __launch_bounds__(2 * WIN * 32)
 ref_scan_kernel(const __nv_bfloat16 *__restrict__ src, const int32_t *__restrict__ seg_lo,
                 const int32_t *__restrict__ seg_hi, float tau, int D,
                 int32_t *__restrict__ src_pos) {
     pdl_enter();
     extern __shared__ uint4 s_buf[];
-    __shared__ float s_dref[kWin], s_dprev[kWin], s_dcur[kWin];   // <w, ref>, <w, w - 1>, <w, s_cur>
-    __shared__ float s_nv[kWin];
+    __shared__ float s_dref[WIN], s_dprev[WIN], s_dcur[WIN];   // <w, ref>, <w, w - 1>, <w, s_cur>
+    __shared__ float s_nv[WIN];
     __shared__ float s_nr;
     __shared__ int s_jr, s_cur, s_w, s_more;   // walk: reference row of the window (-1: entering), row
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int C = D >> 3;
-    uint4 *ref = s_buf + (size_t)kWin * C;
+    uint4 *ref = s_buf + (size_t)WIN * C;
     const int lo = seg_lo[blockIdx.x];
     if (lo < 0) return;
     const int hi = seg_hi[blockIdx.x];
@@ -140,8 +144,8 @@ ref_scan_kernel(const __nv_bfloat16 *__restrict__ src, const int32_t *__restrict
         if (lane == 0) s_nr = nr;
     }
     __syncthreads();
-    for (int j = lo + 1; j < hi; j += kWin) {
-        const int nvalid = hi - j < kWin ? hi - j : kWin;
+    for (int j = lo + 1; j < hi; j += WIN) {
+        const int nvalid = hi - j < WIN ? hi - j : WIN;
         // stage the window's rows (consecutive in src), eight 16-byte loads in flight
         const int total = nvalid * C;
         const uint4 *win = reinterpret_cast<const uint4 *>(src + (int64_t)j * D);
@@ -164,8 +168,8 @@ ref_scan_kernel(const __nv_bfloat16 *__restrict__ src, const int32_t *__restrict
         }
         __syncthreads();
         {
-            const int w = warp < kWin ? warp : warp - kWin;
-            const bool vs_ref = warp < kWin;
+            const int w = warp < WIN ? warp : warp - WIN;
+            const bool vs_ref = warp < WIN;
             if (w < nvalid && (vs_ref || w > 0)) {
                 const uint4 *a = s_buf + (size_t)w * C;
                 float dot, nv;
@@ -606,12 +610,13 @@ RefWs ref_ws(const echo_cache &c, void *ws, int32_t n) {
             reinterpret_cast<int32_t *>(p + 3 * a + b)};
 }
 
-size_t scan_smem_bytes(int D) { return (size_t)(kWin + 1) * D * sizeof(__nv_bfloat16); }
+size_t scan_smem_bytes(int win, int D) { return (size_t)(win + 1) * D * sizeof(__nv_bfloat16); }
 
 // Dynamic shared memory that the scan may ask for on the current device (0: no
 // device): what a CTA may have beside its static buffers.  The kernel's limit is
 // raised to it once per device, whatever the width of the first write there, so that
 // no call depends on the widths written before it or by another thread meanwhile.
+template <int WIN>
 size_t scan_smem_cap() {
     static size_t cap[64] = {};
     static std::mutex mu;
@@ -621,16 +626,23 @@ size_t scan_smem_cap() {
     if (!cap[dev]) {
         cudaFuncAttributes fa;
         int most = 0;
-        if (cudaFuncGetAttributes(&fa, ref_scan_kernel) != cudaSuccess ||
+        if (cudaFuncGetAttributes(&fa, ref_scan_kernel<WIN>) != cudaSuccess ||
             cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
             return 0;
         const int dyn = most - (int)fa.sharedSizeBytes;
-        if (dyn <= 0 || cudaFuncSetAttribute(ref_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (dyn <= 0 || cudaFuncSetAttribute(ref_scan_kernel<WIN>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              dyn) != cudaSuccess)
             return 0;
         cap[dev] = (size_t)dyn;
     }
     return cap[dev];
+}
+
+template <int WIN>
+void launch_scan(const echo_cache &c, const __nv_bfloat16 *src, const RefWs &w, int nseg, cudaStream_t st) {
+    echo::launch_chained(ref_scan_kernel<WIN>, dim3(nseg), dim3(2 * WIN * 32),
+                         scan_smem_bytes(WIN, c.D), st, src, w.seg_lo, w.seg_hi, c.tau, c.D, w.src_pos);
 }
 
 }  // namespace
@@ -684,11 +696,14 @@ echo_status launch_cache_write(const echo_cache &c, const void *src, const int32
     }
     // before anything is enqueued: the release alone would leave slots counted free
     // that the entries still name
-    const size_t scan_smem = scan_smem_bytes(c.D), scan_cap = scan_smem_cap();
-    if (!scan_cap) return ECHO_ERR_CUDA;
-    if (scan_smem > scan_cap) return ECHO_ERR_SHAPE;
     const RefWs w = ref_ws(c, ws, n);
     const int nseg = n_segments(c);
+    const bool wide = nseg <= kWideSegments && scan_smem_bytes(kWinWide, c.D) <= scan_smem_cap<kWinWide>();
+    if (!wide) {
+        const size_t cap = scan_smem_cap<kWin>();
+        if (!cap) return ECHO_ERR_CUDA;
+        if (scan_smem_bytes(kWin, c.D) > cap) return ECHO_ERR_SHAPE;
+    }
     if (cudaMemsetAsync(w.seg_lo, 0xFF, sizeof(int32_t) * (size_t)nseg, st) != cudaSuccess)
         return ECHO_ERR_CUDA;
     {
@@ -699,9 +714,8 @@ echo_status launch_cache_write(const echo_cache &c, const void *src, const int32
     if (last_launch_status() != ECHO_OK) return ECHO_ERR_CUDA;
     {
         LaunchScope ls(ECHO_K_REF_SCAN, n, c.D, 0, st);
-        echo::launch_chained(ref_scan_kernel, dim3(nseg), dim3(kScanWarps * 32), scan_smem, st, s,
-                             w.seg_lo, w.seg_hi, c.tau, c.D,
-                                                             w.src_pos);
+        if (wide) launch_scan<kWinWide>(c, s, w, nseg, st);
+        else launch_scan<kWin>(c, s, w, nseg, st);
     }
     if (last_launch_status() != ECHO_OK) return ECHO_ERR_CUDA;
     {

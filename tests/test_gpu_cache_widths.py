@@ -56,10 +56,21 @@ def test_quant_widths(ec, n, D):
         assert np.array_equal(got[keep], oracle.cache.dequant_gather(oq, os_)[keep])
 
 
-@pytest.mark.parametrize("D", [16, 1024, 1040, 2064, 3504, 5120, 5136, 8192, 8208, 16592])
+@pytest.mark.parametrize("D", [16, 1024, 1040, 2064, 3504, 5120, 5136, 8192, 8208, 8928, 8944, 16592])
 @pytest.mark.parametrize("R_cap", [40, 3])           # 3: runs without a slot, plain int8
 def test_ref_cache_widths(ec, D, R_cap):
-    NT, seg = 60, 20
+    ref_cache(ec, D, R_cap, 60, 20)
+
+
+@pytest.mark.parametrize("NT,seg", [(152 * 14, 14), (153 * 14, 14), (152 * 27 - 5, 27), (500, 3)])
+@pytest.mark.parametrize("D", [16, 320])
+def test_ref_cache_segment_counts(ec, NT, seg, D):
+    """Up to 152 segments the scan takes twelve rows at a time, above six: a whole
+    window, one row more than two, a last segment cut short."""
+    ref_cache(ec, D, NT // 2, NT, seg)
+
+
+def ref_cache(ec, D, R_cap, NT, seg):
     g = ec.DeviceCache(ec.CACHE_REF, NT, D, R_cap=R_cap, seg_len=seg, tau=0.9)
     o = R.RefCache(NT, D, R_cap, seg, 0.9)
     rs = np.random.default_rng(D)
