@@ -16,7 +16,8 @@ SIZES = [
     (257, 192, 192),         # two row tiles, the second of one row; 1.5 column tiles
     (127, 1024, 320),
     (300, 64, 1088),
-    (5000, 128, 2112),       # 256-column tiles, several per pair, the last a quarter wide
+    (5000, 128, 2112),       # 128-column tiles, several per pair, the last half wide
+    (5000, 256, 2112),       # 256-column tiles, several per pair, the last a quarter wide
     (4097, 320, 1600),
 ]
 
